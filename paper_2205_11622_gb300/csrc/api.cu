@@ -116,6 +116,21 @@ struct Layout {
     o_heavy = take(sizeof(HeavyRow) * (size_t)mh);
     o_partial = take(sizeof(float) * (size_t)mc * (size_t)width);
   }
+  // windows of the flat kernels; at most `budget` bytes for the whole layout
+  // (longer windows leave fewer pieces)
+  size_t o_first = 0, o_tail_row = 0, o_pieces = 0;
+  int win = 0, nw = 0;
+  void windows(int64_t nnz, int wm, int width, bool sampled, size_t budget = SIZE_MAX) {
+    const size_t start = cur;
+    for (win = flat_window(nnz, wm, sampled);; win *= 2) {
+      cur = start;
+      nw = (int)((nnz + win - 1) / win);
+      o_first = take(sizeof(int) * (size_t)nw);
+      o_tail_row = take(sizeof(int) * (size_t)nw);
+      o_pieces = take(sizeof(float) * 2 * (size_t)nw * (size_t)width);
+      if (total() <= budget || nw <= 1) return;
+    }
+  }
   size_t o_inter = 0, o_inter2 = 0;
   void inter(size_t bytes) { o_inter = take(bytes); }
   void inter2(size_t bytes) { o_inter2 = take(bytes); }
@@ -137,6 +152,11 @@ SegPlan seg_plan(char* ws, const Layout& l) {
 // The heavy-row records and partial rows of a segment plan, as k_combine reads them.
 SplitPlan combine_plan(const SegPlan& g) {
   return SplitPlan{g.hdr, g.heavy, nullptr, g.partial, g.max_heavy, g.max_chunks};
+}
+
+FlatPlan flat_plan(char* ws, const Layout& l) {
+  return FlatPlan{reinterpret_cast<WsHeader*>(ws), l.win, l.nw, reinterpret_cast<int*>(ws + l.o_first),
+                  reinterpret_cast<int*>(ws + l.o_tail_row), reinterpret_cast<float*>(ws + l.o_pieces)};
 }
 
 UnitPlan unit_plan(char* ws, const Layout& l) {
@@ -221,10 +241,11 @@ slnr_status check_ws(const slnr_opts* o, size_t need) {
   } while (0)
 
 // Zero the header, then (validate mode) run the device check and wait for it.
+// own_header: the call's first kernel sets the only header word that it uses.
 template <typename Launch>
-slnr_status begin(char* ws, cudaStream_t s, bool validate, Launch launch_validate) {
+slnr_status begin(char* ws, cudaStream_t s, bool validate, Launch launch_validate, bool own_header = false) {
   WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
-  SLNR_CUDA(cudaMemsetAsync(hdr, 0, sizeof(WsHeader), s));
+  if (!own_header || validate) SLNR_CUDA(cudaMemsetAsync(hdr, 0, sizeof(WsHeader), s));
   if (validate) {
     SLNR_CUDA(launch_validate(hdr));
     int flag = 0;
@@ -276,12 +297,36 @@ Layout layout_spmm_gemm(const slnr_csr* B, int32_t K, int32_t L, const slnr_opts
   return l;
 }
 
-Layout layout_sddmm_spmm(const slnr_csr* B, int32_t L, int32_t K, int variant) {
-  (void)L;
+// Fused <SDDMM,SpMM> runs on the nonzero-window kernels, whatever the widths,
+// but for large calls and short rows at widths of powers of two up to 64:
+// there four or more windows share a warp, short rows start in one or another
+// of them at almost every step, and the row kernel (a lane group per short
+// row) is ahead (us, windows | rows: R-MAT 5.1M nonzeros 64/64 367 | 342,
+// 14.5M 64/32 720 | 652, 117k rows of 3.1 64/64 72 | 66; otherwise 3.7M 64/32
+// 160 | 160, 2.0M 64/64 120 | 133; wider, 4.8M 128/128 327 | 391).
+constexpr int64_t kRowsMinNnz = int64_t(1) << 22;
+bool use_flat_sddmm(int64_t nrows, int64_t nnz, int32_t L, int32_t K) {
+  return (nnz < kRowsMinNnz && nnz >= 4 * nrows) || L > 64 || K > 64 || !all_pow2(L, K);
+}
+
+Layout layout_sddmm_spmm(const slnr_csr* B, int32_t L, int32_t K, int variant, size_t budget = SIZE_MAX) {
   Layout l;
-  l.split(B->nrows, B->nnz, K);
-  if (variant == SLNR_UNFUSED) l.inter(sizeof(float) * (size_t)B->nnz);
+  if (variant == SLNR_FUSED && use_flat_sddmm(B->nrows, B->nnz, L, K)) {
+    l.windows(B->nnz, L > K ? L : K, K, true, budget);
+  } else {
+    l.split(B->nrows, B->nnz, K);
+    if (variant == SLNR_UNFUSED) l.inter(sizeof(float) * (size_t)B->nnz);
+  }
   return l;
+}
+
+// Fused <SDDMM,SpMM> on the nonzero-window kernels.
+slnr_status flat_sddmm_spmm(const CsrView& v, const float* C, const float* D, int32_t L, const float* E, int32_t K,
+                            float* A, char* ws, const Layout& l, cudaStream_t s) {
+  const FlatPlan fp = flat_plan(ws, l);
+  SLNR_LAUNCH("flat_rows", launch_flat_rows(v, K, A, fp, s));
+  SLNR_LAUNCH("flat_sddmm_spmm", launch_flat_sampled(v, C, D, L, E, K, A, fp, s));
+  return SLNR_OK;
 }
 
 Layout layout_mttkrp(const slnr_csf3* B, int32_t L, int variant) {
@@ -397,7 +442,69 @@ slnr_status wide_mttkrp(const slnr_csf3* B, const float* C, const float* D, int3
   return SLNR_OK;
 }
 
+// <SDDMM,SpMM>; fused, in at most `budget` bytes of workspace.
+slnr_status sddmm_spmm(const slnr_csr* B, const float* C, const float* D, int32_t L, const float* E, int32_t K,
+                       float* A, const slnr_opts* opts, size_t budget) {
+  g_last_error[0] = '\0';
+  timing_begin();
+  SLNR_CHECK(check_opts(opts));
+  SLNR_CHECK(check_csr(B, true));
+  SLNR_CHECK(check_dims("L", L));
+  SLNR_CHECK(check_dims("K", K));
+  SLNR_CHECK(check_dense("C", C));
+  SLNR_CHECK(check_dense("D", D));
+  SLNR_CHECK(check_dense("E", E));
+  SLNR_CHECK(check_dense("A", A));
+  const Layout l = layout_sddmm_spmm(B, L, K, opts->variant, budget);
+  SLNR_CHECK(check_ws(opts, l.total()));
+  if (B->nrows == 0) return SLNR_OK;
+  cudaStream_t s = static_cast<cudaStream_t>(opts->stream);
+  char* ws = static_cast<char*>(opts->workspace);
+  const bool flat = opts->variant == SLNR_FUSED && use_flat_sddmm(B->nrows, B->nnz, L, K);
+  SLNR_CHECK(begin(ws, s, opts->validate != 0,
+                   [&](WsHeader* h) { return launch_validate_csr(*B, h, s); }, flat));
+  const CsrView v = csr_view(B);
+  if (flat) {
+    SLNR_CHECK(flat_sddmm_spmm(v, C, D, L, E, K, A, ws, l, s));
+    return finish(ws, s, opts->validate != 0);
+  }
+  const SplitPlan sp = split_plan(ws, l);
+  SLNR_LAUNCH("classify", launch_classify(v, sp, s));
+  if (!all_pow2(L, K)) {
+    float* Y = reinterpret_cast<float*>(ws + l.o_inter);
+    SLNR_LAUNCH("w_sddmm", launch_w_sddmm_spmm(v, C, D, L, nullptr, K, nullptr, Y, sp, s));
+    CsrView vy = v;
+    vy.vals = Y;
+    SLNR_LAUNCH("w_spmm", launch_w_spmm(K, vy, E, nullptr, A, sp, s));
+    SLNR_LAUNCH("w_combine", launch_w_combine(K, sp, nullptr, 0, A, s));
+  } else if (opts->variant == SLNR_FUSED) {
+    SLNR_LAUNCH("sddmm_spmm_rows", launch_sddmm_spmm_rows(v, C, D, L, E, K, A, sp, s));
+    SLNR_LAUNCH("combine", launch_combine(K, sp, nullptr, 0, A, s));
+  } else {
+    float* Y = reinterpret_cast<float*>(ws + l.o_inter);
+    SLNR_LAUNCH("sddmm_rows", launch_sddmm_rows(v, C, D, L, Y, s));
+    SLNR_LAUNCH("sddmm_chunks", launch_sddmm_chunks(v, C, D, L, Y, sp, s));
+    CsrView vy = v;
+    vy.vals = Y;
+    SLNR_LAUNCH("spmm_chunks", launch_spmm_chunks(K, vy, E, sp, s));
+    SLNR_LAUNCH("spmm_rows", launch_spmm_rows(K, vy, E, A, s));
+    SLNR_LAUNCH("combine", launch_combine(K, sp, nullptr, 0, A, s));
+  }
+  return finish(ws, s, opts->validate != 0);
+}
+
 }  // namespace
+
+size_t slnr::split_scratch_bytes(const slnr_csr& B, int32_t K) {
+  Layout l;
+  l.split(B.nrows, B.nnz, K);
+  return l.total();
+}
+
+slnr_status slnr::sddmm_spmm_within(const slnr_csr* B, const float* C, const float* D, int32_t L, const float* E,
+                                    int32_t K, float* A, const slnr_opts* opts) {
+  return sddmm_spmm(B, C, D, L, E, K, A, opts, opts->workspace_bytes);
+}
 
 void slnr::set_last_error(const char* msg) { snprintf(g_last_error, sizeof(g_last_error), "%s", msg); }
 
@@ -606,51 +713,7 @@ slnr_status slnr_spmm_gemm(const slnr_csr* B, const float* C, int32_t K, const f
 
 slnr_status slnr_sddmm_spmm(const slnr_csr* B, const float* C, const float* D, int32_t L, const float* E,
                             int32_t K, float* A, const slnr_opts* opts) {
-  g_last_error[0] = '\0';
-  timing_begin();
-  SLNR_CHECK(check_opts(opts));
-  SLNR_CHECK(check_csr(B, true));
-  SLNR_CHECK(check_dims("L", L));
-  SLNR_CHECK(check_dims("K", K));
-  SLNR_CHECK(check_dense("C", C));
-  SLNR_CHECK(check_dense("D", D));
-  SLNR_CHECK(check_dense("E", E));
-  SLNR_CHECK(check_dense("A", A));
-  const Layout l = layout_sddmm_spmm(B, L, K, opts->variant);
-  SLNR_CHECK(check_ws(opts, l.total()));
-  if (B->nrows == 0) return SLNR_OK;
-  cudaStream_t s = static_cast<cudaStream_t>(opts->stream);
-  char* ws = static_cast<char*>(opts->workspace);
-  SLNR_CHECK(begin(ws, s, opts->validate != 0,
-                   [&](WsHeader* h) { return launch_validate_csr(*B, h, s); }));
-  const CsrView v = csr_view(B);
-  const SplitPlan sp = split_plan(ws, l);
-  SLNR_LAUNCH("classify", launch_classify(v, sp, s));
-  if (!all_pow2(L, K)) {
-    if (opts->variant == SLNR_FUSED) {
-      SLNR_LAUNCH("w_sddmm_spmm", launch_w_sddmm_spmm(v, C, D, L, E, K, A, nullptr, sp, s));
-    } else {
-      float* Y = reinterpret_cast<float*>(ws + l.o_inter);
-      SLNR_LAUNCH("w_sddmm", launch_w_sddmm_spmm(v, C, D, L, nullptr, K, nullptr, Y, sp, s));
-      CsrView vy = v;
-      vy.vals = Y;
-      SLNR_LAUNCH("w_spmm", launch_w_spmm(K, vy, E, nullptr, A, sp, s));
-    }
-    SLNR_LAUNCH("w_combine", launch_w_combine(K, sp, nullptr, 0, A, s));
-  } else if (opts->variant == SLNR_FUSED) {
-    SLNR_LAUNCH("sddmm_spmm_rows", launch_sddmm_spmm_rows(v, C, D, L, E, K, A, sp, s));
-    SLNR_LAUNCH("combine", launch_combine(K, sp, nullptr, 0, A, s));
-  } else {
-    float* Y = reinterpret_cast<float*>(ws + l.o_inter);
-    SLNR_LAUNCH("sddmm_rows", launch_sddmm_rows(v, C, D, L, Y, s));
-    SLNR_LAUNCH("sddmm_chunks", launch_sddmm_chunks(v, C, D, L, Y, sp, s));
-    CsrView vy = v;
-    vy.vals = Y;
-    SLNR_LAUNCH("spmm_chunks", launch_spmm_chunks(K, vy, E, sp, s));
-    SLNR_LAUNCH("spmm_rows", launch_spmm_rows(K, vy, E, A, s));
-    SLNR_LAUNCH("combine", launch_combine(K, sp, nullptr, 0, A, s));
-  }
-  return finish(ws, s, opts->validate != 0);
+  return sddmm_spmm(B, C, D, L, E, K, A, opts, SIZE_MAX);
 }
 
 slnr_status slnr_mttkrp(const slnr_csf3* B, const float* C, const float* D, int32_t L, float* A,

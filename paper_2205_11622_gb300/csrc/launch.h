@@ -60,6 +60,16 @@ struct SegPlan {
   int max_chunks;
 };
 
+// Workspace pieces of the nonzero-window kernels (flat.cu).
+struct FlatPlan {
+  WsHeader* hdr;
+  int win;        // nonzeros per window (flat_window)
+  int nw;         // windows: ceil(nnz / win)
+  int* first;     // [nw]
+  int* tail_row;  // [nw]
+  float* pieces;  // 2 x nw rows of the output width: heads, then tails
+};
+
 int device_sm_count();
 
 // Sets the calling thread's slnr_last_error() text (api.cu).
@@ -114,6 +124,21 @@ bool tc_sampled_supported(int K, int L, int M);
 cudaError_t launch_tc_sddmm_spmm_gemm(const CsrView& B, const float* C, const float* D, const float* F, int L,
                                       const float* W, int M, float* A, const SegPlan& plan, cudaStream_t s);
 
+// flat.cu -- row sums over windows of consecutive nonzeros, any width up to
+// kWideMax, in two steps of a call: launch_flat_rows (zeroes the rows without
+// nonzeros and the header's flag word), then the sums; together they write
+// every row of out (width W or K).
+// Window length for nnz nonzeros and gathered rows of at most wm values
+// (sampled: for launch_flat_sampled).
+int flat_window(int64_t nnz, int wm, bool sampled);
+cudaError_t launch_flat_rows(const CsrView& B, int W, float* out, const FlatPlan& plan, cudaStream_t s);
+// out = B . X (with X2 not NULL the gathered row is X .* X2)
+cudaError_t launch_flat_sum(const CsrView& B, const float* X, const float* X2, int W, float* out, const FlatPlan& plan,
+                            cudaStream_t s);
+// fused <SDDMM,SpMM>: C nrows x L, D ncols x L, E ncols x K
+cudaError_t launch_flat_sampled(const CsrView& B, const float* C, const float* D, int L, const float* E, int K,
+                                float* out, const FlatPlan& plan, cudaStream_t s);
+
 // sddmm.cu
 // fused <SDDMM,SpMM>: the heavy rows' chunks (partials) and the light rows in
 // one launch (plan.hdr->next_row must be 0: warps take work from it)
@@ -138,6 +163,12 @@ cudaError_t launch_mttkrp_stage2_units(int L, const slnr_csf3& B, const float* T
 // that sum times E (A has width M).
 cudaError_t launch_mttkrp_combine(int L, const slnr_csf3& B, const UnitPlan& plan, const float* E, int M,
                                   float* A, cudaStream_t s);
+
+// api.cu -- the size that a heavy-row split of B takes (what the built-in scratch is measured by), and
+// slnr_sddmm_spmm (fused) with windows long enough to fit opts->workspace_bytes
+size_t split_scratch_bytes(const slnr_csr& B, int32_t K);
+slnr_status sddmm_spmm_within(const slnr_csr* B, const float* C, const float* D, int32_t L, const float* E, int32_t K,
+                              float* A, const slnr_opts* opts);
 
 // wide.cu -- any inner width that is a multiple of 4 up to kWideMax, chosen at
 // run time (the kernels above take powers of two in [4, 256])

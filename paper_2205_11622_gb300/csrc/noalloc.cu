@@ -65,6 +65,9 @@ extern "C" slnr_status slnr_sddmm_spmm_noalloc(const slnr_csr* B, const float* C
   size_t need = 0;
   slnr_status st = slnr_sddmm_spmm_workspace(B, L, K, &o, &need);
   if (st != SLNR_OK) return st;
+  // the sizes accepted are those whose heavy-row split fits (a bound of nnz,
+  // rows and K); the windows of the call are then made long enough to fit
+  need = slnr::split_scratch_bytes(*B, K);
   if (need > kNoAllocScratchBytes) {
     char msg[256];
     snprintf(msg, sizeof(msg),
@@ -84,5 +87,5 @@ extern "C" slnr_status slnr_sddmm_spmm_noalloc(const slnr_csr* B, const float* C
   }
   o.workspace = scratch;
   o.workspace_bytes = kNoAllocScratchBytes;
-  return slnr_sddmm_spmm(B, C, D, L, E, K, A, &o);
+  return slnr::sddmm_spmm_within(B, C, D, L, E, K, A, &o);
 }
