@@ -275,6 +275,7 @@ slnr_status finish(char* ws, cudaStream_t s, bool validate) {
 // ---------------------------------------------------------------------------
 // layouts per operation
 
+
 // The fused tensor-core path takes row segments; everything else splits heavy rows.
 bool use_tc(const slnr_opts* o, int32_t K, int32_t L) { return o->allow_tf32 != 0 && tc_supported(K, L); }
 
@@ -286,8 +287,60 @@ bool use_tc_fused(const slnr_opts* o, int32_t K, int32_t L, int64_t nnz) {
   return o->variant == SLNR_FUSED && use_tc(o, K, L) && nnz >= kTcFusedMinNnz;
 }
 
-Layout layout_spmm_gemm(const slnr_csr* B, int32_t K, int32_t L, const slnr_opts* o) {
+// Which contraction of A = B.X.D comes first (X a gathered matrix, X .* X2 in
+// <SpMMH,GEMM>, F and W in <SDDMM,SpMM,GEMM>).  Row first: T = B.X row by row
+// on chip, T.D at once (nnz K gathered values, nrows K L products).  D first:
+// G = X.D once per row of X into the workspace, then A = B.G summed straight
+// into its rows (flat.cu: nnz L gathered values, ncols K L products, G written
+// and read through L2).  The sums are the same ones in another order; the
+// tensor cores then round D only (X goes in as two tf32 parts), so the error
+// against 64 bits is smaller (3.0e-4 -> 2.1e-4; without them both are fp32).
+//
+// Measured on R-MAT graphs of 3k to 1M rows at degrees 4 to 16 and tensors of
+// 60k to 20M nonzeros (us, row first | D first):
+//  - fp32, or widths without a tensor-core row kernel: D first throughout
+//    (150k rows 64/32 295 | 110, 50k rows 100/48 148 | 71, 500k 64/64 588 |
+//    246), unless D widens the rows more than four times on a call of some
+//    size (uniform 220k rows 12/256 158 | 307);
+//  - fibers (<SpTTM,SpTTM>): D first (20M nonzeros 64/64 712 | 430, 1M 156 | 82);
+//  - tensor cores: D first on graphs of fewer rows, where the row kernel's
+//    tiles of heavy rows set its time (50k rows 128/128 159 | 90, 220k 64/64
+//    201 | 128), row first on larger ones (500k 32/32 118 | 160, 1M 128/128
+//    940 | 1000) and where D widens the rows (220k 32/128 107 | 154); two
+//    gathered matrices move the line up (1M 128/128 1750 | 1077).
+bool use_tc_premul(const slnr_opts* o, int32_t K, int32_t L, int64_t nnz) {
+  return o->allow_tf32 != 0 && tc_split_supported(K, L) && nnz >= kTcFusedMinNnz;
+}
+enum PremulKind { kOne, kTwo, kSampledRows, kFibers };
+bool premul_first(const slnr_opts* o, PremulKind kind, int64_t nrows, int64_t ncols, int64_t nnz, int32_t K, int32_t L,
+                  bool row_tc) {
+  if (o->variant != SLNR_FUSED || nnz < 1 || nnz < ncols) return false;
+  if (L > K && nnz > 64 * nrows) return false;  // long rows: the narrower rows are gathered
+  if (kind == kFibers) return true;
+  if (!row_tc) return L <= 4 * K || nnz < (int64_t(1) << 18);
+  const int64_t k = 1024, few = (K <= 32 ? 128 : 256) * k;
+  if (L > 2 * K) return nrows < 64 * k;
+  if (kind == kTwo) return nrows < few || nnz >= 8 * nrows;
+  if (nrows >= few) return kind == kOne && K == 64 && L < 64 && nnz >= 8 * nrows;
+  return K < 128 || nrows < 64 * k || nnz >= 8 * nrows;
+}
+
+// Workspace of the premultiplied order: G (ncols x L), then the windows.
+Layout layout_premul(int64_t ncols, int64_t nnz, int wm, int32_t L, bool sampled) {
   Layout l;
+  l.windows(nnz, wm, L, sampled);
+  l.inter(sizeof(float) * (size_t)ncols * (size_t)L);
+  return l;
+}
+
+bool premul_spmm(const slnr_csr* B, int32_t K, int32_t L, const slnr_opts* o, bool two) {
+  return premul_first(o, two ? kTwo : kOne, B->nrows, B->ncols, B->nnz, K, L, use_tc_fused(o, K, L, B->nnz));
+}
+
+// (two: <SpMMH,GEMM>, two gathered matrices)
+Layout layout_spmm_gemm(const slnr_csr* B, int32_t K, int32_t L, const slnr_opts* o, bool two = false) {
+  Layout l;
+  if (premul_spmm(B, K, L, o, two)) return layout_premul(B->ncols, B->nnz, L, L, false);
   if (use_tc_fused(o, K, L, B->nnz)) {
     l.segs(B->nrows, B->nnz, L);
   } else {
@@ -339,8 +392,13 @@ Layout layout_mttkrp(const slnr_csf3* B, int32_t L, int variant) {
   return l;
 }
 
+bool premul_spttm(const slnr_csf3* B, int32_t L, int32_t M, const slnr_opts* o) {
+  return premul_first(o, kFibers, B->nfibers, B->dim[2], B->nnz, L, M, false);
+}
+
 Layout layout_spttm_ttm(const slnr_csf3* B, int32_t L, int32_t M, const slnr_opts* o) {
   Layout l;
+  if (premul_spttm(B, L, M, o)) return layout_premul(B->dim[2], B->nnz, M, M, false);
   if (use_tc_fused(o, L, M, B->nnz)) {
     l.segs(B->nfibers, B->nnz, M);
   } else {
@@ -356,9 +414,15 @@ bool use_tc_sampled(const slnr_opts* o, int32_t K, int32_t L, int32_t M, int64_t
   return o->variant == SLNR_FUSED && o->allow_tf32 != 0 && tc_sampled_supported(K, L, M) && nnz >= kTcFusedMinNnz;
 }
 
+bool premul_sampled(const slnr_csr* B, int32_t K, int32_t L, int32_t M, const slnr_opts* o) {
+  return premul_first(o, kSampledRows, B->nrows, B->ncols, B->nnz, L, M, use_tc_sampled(o, K, L, M, B->nnz));
+}
+
 Layout layout_sddmm_spmm_gemm(const slnr_csr* B, int32_t K, int32_t L, int32_t M, const slnr_opts* o) {
   const int variant = o->variant;
   Layout l;
+  if (premul_sampled(B, K, L, M, o))
+    return layout_premul(B->ncols, B->nnz, K > M ? K : M, M, true);
   if (use_tc_sampled(o, K, L, M, B->nnz)) {
     l.segs(B->nrows, B->nnz, M);
     return l;
@@ -385,6 +449,29 @@ Layout layout_mttkrp_gemm(const slnr_csf3* B, int32_t L, int variant) {
 CsrView csr_view(const slnr_csr* B) { return CsrView{B->nrows, B->ncols, B->nnz, B->pos, B->crd, B->vals}; }
 CsrView fiber_view(const slnr_csf3* B) {
   return CsrView{B->nfibers, B->dim[2], B->nnz, B->pos3, B->crd3, B->vals};
+}
+
+// G = X . D or (X .* X2) . D into the workspace, on the tensor cores where allowed.
+slnr_status premul(int64_t ncols, int32_t K, int32_t L, const float* X, const float* X2, const float* D, float* G,
+                   char* ws, bool tc, cudaStream_t s) {
+  if (tc)
+    SLNR_LAUNCH("tc_premul", launch_tc_premul(ncols, K, L, X, X2, D, G, reinterpret_cast<WsHeader*>(ws), s));
+  else
+    SLNR_LAUNCH("premul", launch_premul(ncols, K, L, X, X2, D, G, s));
+  return SLNR_OK;
+}
+
+// A = B . G with G = X . D (or (X .* X2) . D): the consumer's contraction once
+// per row of X, then the rows of G summed (flat.cu).
+slnr_status premul_sum(const CsrView& v, const float* X, const float* X2, int32_t K, const float* D, int32_t L,
+                       float* A, char* ws, const Layout& l, bool tc, cudaStream_t s) {
+  float* G = reinterpret_cast<float*>(ws + l.o_inter);
+  FlatPlan fp = flat_plan(ws, l);
+  if (tc) fp.hdr = nullptr;  // zeroed before the tensor-core kernel, which may raise a flag
+  SLNR_CHECK(premul(v.ncols, K, L, X, X2, D, G, ws, tc, s));
+  SLNR_LAUNCH("flat_rows", launch_flat_rows(v, L, A, fp, s));
+  SLNR_LAUNCH("flat_sum", launch_flat_sum(v, G, nullptr, L, A, fp, s));
+  return SLNR_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -659,7 +746,7 @@ slnr_status slnr_spmmh_gemm_workspace(const slnr_csr* B, int32_t J, int32_t L, c
   SLNR_CHECK(check_dims("J", J));
   SLNR_CHECK(check_dims("L", L));
   if (!bytes) return fail(SLNR_ERR_NULL, "bytes is NULL");
-  *bytes = layout_spmm_gemm(B, J, L, opts).total();
+  *bytes = layout_spmm_gemm(B, J, L, opts, true).total();
   return SLNR_OK;
 }
 
@@ -679,11 +766,14 @@ slnr_status slnr_spmm_gemm(const slnr_csr* B, const float* C, int32_t K, const f
   if (B->nrows == 0) return SLNR_OK;
   cudaStream_t s = static_cast<cudaStream_t>(opts->stream);
   char* ws = static_cast<char*>(opts->workspace);
+  const bool pre = premul_spmm(B, K, L, opts, false), pre_tc = use_tc_premul(opts, K, L, B->nnz);
   SLNR_CHECK(begin(ws, s, opts->validate != 0,
-                   [&](WsHeader* h) { return launch_validate_csr(*B, h, s); }));
+                   [&](WsHeader* h) { return launch_validate_csr(*B, h, s); }, pre && !pre_tc));
   const CsrView v = csr_view(B);
   const bool tc = use_tc(opts, K, L);
-  if (use_tc_fused(opts, K, L, B->nnz)) {
+  if (pre) {
+    SLNR_CHECK(premul_sum(v, C, nullptr, K, D, L, A, ws, l, pre_tc, s));
+  } else if (use_tc_fused(opts, K, L, B->nnz)) {
     const SegPlan gp = seg_plan(ws, l);
     SLNR_LAUNCH("seg_count", launch_seg_count(v, gp, s));
     SLNR_LAUNCH("seg_write", launch_seg_write(v, gp, s));
@@ -773,14 +863,17 @@ slnr_status slnr_spttm_ttm(const slnr_csf3* B, const float* C, int32_t L, const 
   SLNR_CHECK(check_ws(opts, l.total()));
   cudaStream_t s = static_cast<cudaStream_t>(opts->stream);
   char* ws = static_cast<char*>(opts->workspace);
+  const bool pre = premul_spttm(B, L, M, opts), pre_tc = use_tc_premul(opts, L, M, B->nnz);
   SLNR_CHECK(begin(ws, s, opts->validate != 0,
-                   [&](WsHeader* h) { return launch_validate_csf(*B, h, s); }));
+                   [&](WsHeader* h) { return launch_validate_csf(*B, h, s); }, pre && !pre_tc));
   // A's two compressed levels are B's (the (i,j) pattern is unchanged)
   SLNR_LAUNCH("copy_levels", launch_copy_levels(*B, A_pos1, A_crd1, A_pos2, A_crd2, s));
   if (B->nfibers == 0) return SLNR_OK;
   const CsrView fv = fiber_view(B);
   const bool tc = use_tc(opts, L, M);
-  if (use_tc_fused(opts, L, M, B->nnz)) {
+  if (pre) {
+    SLNR_CHECK(premul_sum(fv, C, nullptr, L, D, M, A_vals, ws, l, pre_tc, s));
+  } else if (use_tc_fused(opts, L, M, B->nnz)) {
     const SegPlan gp = seg_plan(ws, l);
     SLNR_LAUNCH("seg_count", launch_seg_count(fv, gp, s));
     SLNR_LAUNCH("seg_write", launch_seg_write(fv, gp, s));
@@ -827,9 +920,20 @@ slnr_status slnr_sddmm_spmm_gemm(const slnr_csr* B, const float* C, const float*
   if (B->nrows == 0) return SLNR_OK;
   cudaStream_t s = static_cast<cudaStream_t>(opts->stream);
   char* ws = static_cast<char*>(opts->workspace);
+  const bool pre = premul_sampled(B, K, L, M, opts), pre_tc = use_tc_premul(opts, L, M, B->nnz);
   SLNR_CHECK(begin(ws, s, opts->validate != 0,
-                   [&](WsHeader* h) { return launch_validate_csr(*B, h, s); }));
+                   [&](WsHeader* h) { return launch_validate_csr(*B, h, s); }, pre && !pre_tc));
   const CsrView v = csr_view(B);
+  if (pre) {
+    // F . W once, then <SDDMM,SpMM> over its rows
+    float* G = reinterpret_cast<float*>(ws + l.o_inter);
+    FlatPlan fp = flat_plan(ws, l);
+    if (pre_tc) fp.hdr = nullptr;
+    SLNR_CHECK(premul(v.ncols, L, M, F, nullptr, W, G, ws, pre_tc, s));
+    SLNR_LAUNCH("flat_rows", launch_flat_rows(v, M, A, fp, s));
+    SLNR_LAUNCH("flat_sddmm_spmm", launch_flat_sampled(v, C, D, K, G, M, A, fp, s));
+    return finish(ws, s, opts->validate != 0);
+  }
   if (use_tc_sampled(opts, K, L, M, B->nnz)) {
     // T(i,:) built on chip by the producers, T.W on the TF32 tensor cores;
     // heavy rows' chunk rows of A are summed by the combine
@@ -940,18 +1044,21 @@ slnr_status slnr_spmmh_gemm(const slnr_csr* B, const float* C, const float* D, i
   SLNR_CHECK(check_dense("D", D));
   SLNR_CHECK(check_dense("E", E));
   SLNR_CHECK(check_dense("A", A));
-  const Layout l = layout_spmm_gemm(B, J, L, opts);
+  const Layout l = layout_spmm_gemm(B, J, L, opts, true);
   SLNR_CHECK(check_ws(opts, l.total()));
   if (B->nrows == 0) return SLNR_OK;
   cudaStream_t s = static_cast<cudaStream_t>(opts->stream);
   char* ws = static_cast<char*>(opts->workspace);
+  const bool pre = premul_spmm(B, J, L, opts, true), pre_tc = use_tc_premul(opts, J, L, B->nnz);
   SLNR_CHECK(begin(ws, s, opts->validate != 0,
-                   [&](WsHeader* h) { return launch_validate_csr(*B, h, s); }));
+                   [&](WsHeader* h) { return launch_validate_csr(*B, h, s); }, pre && !pre_tc));
   const CsrView v = csr_view(B);
   const bool tc = use_tc(opts, J, L);
   const bool tc_fused = use_tc_fused(opts, J, L, B->nnz);
   // the gathered row of column k is C(k,:) .* D(k,:); E is the consumer matrix
-  if (tc_fused) {
+  if (pre) {
+    SLNR_CHECK(premul_sum(v, C, D, J, E, L, A, ws, l, pre_tc, s));
+  } else if (tc_fused) {
     const SegPlan gp = seg_plan(ws, l);
     SLNR_LAUNCH("seg_count", launch_seg_count(v, gp, s));
     SLNR_LAUNCH("seg_write", launch_seg_write(v, gp, s));

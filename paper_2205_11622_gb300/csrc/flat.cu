@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(kRowsThreads) k_flat_rows(const FlatArgs a) {
   const int lane = threadIdx.x & 31;
   const int64_t r0 = ((int64_t)blockIdx.x * kRowsThreads + threadIdx.x) - lane, r = r0 + lane;
   flat::grid_launch();
-  if (blockIdx.x == 0 && threadIdx.x == 0) a.hdr->error = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0 && a.hdr != nullptr) a.hdr->error = 0;
   const bool in = r < a.nrows;
   const int p0 = in ? __ldg(a.pos + r) : 0, p1 = in ? __ldg(a.pos + r + 1) : 0;
   int w0 = 0, w1 = 0;
@@ -525,8 +525,10 @@ int flat_window(int64_t nnz, int wm, bool sampled) {
   int64_t k = nnz / (groups * 6 * 2 * gs);
   const int64_t most = gs >= 16 ? (sampled ? 7 : 3) : sampled ? 2 : 9;
   if (k > most) k = most;
-  if (k < 1) k = 1;
-  if (most > 2) k -= (k + 1) % 2;
+  // at least 16 nonzeros, but for calls too small to fill the GPU with them
+  const int64_t least = nnz < (int64_t(1) << 17) || gs >= 8 ? 1 : 16 / (2 * gs);
+  if (k < least) k = least;
+  if (most > 2 && k > 1) k += (k + 1) % 2;
   return (int)k * 2 * gs;
 }
 

@@ -62,7 +62,7 @@ struct SegPlan {
 
 // Workspace pieces of the nonzero-window kernels (flat.cu).
 struct FlatPlan {
-  WsHeader* hdr;
+  WsHeader* hdr;  // its flag word is zeroed by the call's first kernel (NULL: the call has zeroed the header)
   int win;        // nonzeros per window (flat_window)
   int nw;         // windows: ceil(nnz / win)
   int* first;     // [nw]
@@ -118,6 +118,11 @@ cudaError_t launch_tc_spmm_gemm(int K, int L, const CsrView& B, const float* C, 
                                 const SegPlan& plan, cudaStream_t s, const float* C2 = nullptr);
 cudaError_t launch_tc_dense_gemm(int64_t M, int K, int L, const float* T, const float* D, float* A,
                                  WsHeader* hdr, cudaStream_t s);
+// G = X . D, or (X .* X2) . D (X, X2: M x K, D: K x L): X in two tf32 parts,
+// D rounded to tf32 (hdr zeroed by the call: the kernel takes tiles from it)
+bool tc_split_supported(int K, int L);
+cudaError_t launch_tc_premul(int64_t M, int K, int L, const float* X, const float* X2, const float* D, float* G,
+                             WsHeader* hdr, cudaStream_t s);
 // fused <SDDMM,SpMM,GEMM> on the tensor-core kernel: C nrows x K, D ncols x K,
 // F ncols x L, W L x M, with K == L (the dot product and the temporary share the lane layout)
 bool tc_sampled_supported(int K, int L, int M);
@@ -138,6 +143,10 @@ cudaError_t launch_flat_sum(const CsrView& B, const float* X, const float* X2, i
 // fused <SDDMM,SpMM>: C nrows x L, D ncols x L, E ncols x K
 cudaError_t launch_flat_sampled(const CsrView& B, const float* C, const float* D, int L, const float* E, int K,
                                 float* out, const FlatPlan& plan, cudaStream_t s);
+
+// premul.cu -- the same in fp32 on the CUDA cores, any widths
+cudaError_t launch_premul(int64_t M, int K, int L, const float* X, const float* X2, const float* D, float* G,
+                          cudaStream_t s);
 
 // sddmm.cu
 // fused <SDDMM,SpMM>: the heavy rows' chunks (partials) and the light rows in

@@ -82,3 +82,57 @@ def test_sddmm_spmm_windows(slnr, L, K, kind):
 def shifted(t, n=4):
     """A contiguous copy of t that starts n elements into its storage."""
     return torch.cat([t.new_zeros(n), t.reshape(-1)])[n:].view(t.shape)
+
+
+@pytest.mark.parametrize("J,L", [(8, 8), (16, 4), (32, 16), (24, 20), (64, 64), (128, 96), (256, 256), (512, 300), (36, 36)])
+@pytest.mark.parametrize("kind", ["window_ends", "long", "empty_runs"])
+@pytest.mark.parametrize("op", ["spmm_gemm", "spmmh_gemm"])
+def test_premultiplied_sums(slnr, op, J, L, kind):
+    # A = B . (X . D): the contraction once per column of B (both in fp32 and,
+    # where the widths allow, with X in two tf32 parts), then sums over windows
+    rng = np.random.default_rng(J + L)
+    lens = structure(kind, rng)
+    ncols = {"empty_runs": 45, "window_ends": 2000, "long": 9100}[kind]
+    lens = [min(n, ncols) for n in lens]
+    B = csr(lens, ncols, rng, 0x51A4 + J)
+    r = wl.Rng(0x51A4 + 7 * L)
+    names = ("C", "D") if op == "spmm_gemm" else ("C", "D", "E")
+    dense = {k: wl.uniform(r, (ncols, J), -1, 1) for k in names[:-1]}
+    dense[names[-1]] = wl.uniform(r, (J, L), -1, 1)
+    w = wl.Workload(kind, op, B, dense, {"K": J, "J": J, "L": L})
+    ref, ref_abs = oracle.get().run(w)
+    dB, dd = P.to_device(w)
+    for tf32 in (False, True):
+        out = torch.full((B.nrows, L), float("nan"), device="cuda")
+        slnr.timing_enable(True)
+        try:
+            slnr.run(op, dB, dd, out=out, allow_tf32=tf32)
+            names = [n for n, _ in slnr.timing_read()]
+        finally:
+            slnr.timing_enable(False)
+        assert "flat_sum" in names, names
+        assert slnr.device_flags() == 0
+        assert P.rel_err(out.cpu().numpy(), ref, ref_abs) <= P.tolerance(op, tf32)
+
+
+@pytest.mark.parametrize("K,L", [(16, 16), (32, 128), (64, 64), (128, 128), (128, 16)])
+@pytest.mark.parametrize("two", [False, True])
+def test_split_product_error(slnr, K, L, two):
+    # X enters the tensor cores as two tf32 parts, so only D's rounding is left:
+    # with D exactly representable in tf32 the result is as good as fp32's
+    # (2^-22 from the parts and K 2^-24 from the sums, well below 1e-5)
+    n = 700
+    r = wl.Rng(0x51A4 + K + L)
+    B = wl.CSR(n, n, np.arange(n + 1, dtype=np.int32) * 30, np.concatenate(
+        [np.sort(np.random.default_rng(i).choice(n, 30, replace=False)) for i in range(n)]).astype(np.int32),
+        wl.uniform(r, 30 * n, -1, 1))
+    D = np.round(wl.uniform(r, (K, L), -1, 1) * 512).astype(np.float32) / 512
+    if two:
+        w = wl.Workload("split", "spmmh_gemm", B, {"C": wl.uniform(r, (n, K), -1, 1), "D": wl.uniform(r, (n, K), -1, 1),
+                                                   "E": D}, {"J": K, "L": L})
+    else:
+        w = wl.Workload("split", "spmm_gemm", B, {"C": wl.uniform(r, (n, K), -1, 1), "D": D}, {"K": K, "L": L})
+    ref, ref_abs = oracle.get().run(w)
+    dB, dd = P.to_device(w)
+    out = slnr.run(w.op, dB, dd, allow_tf32=True)
+    assert P.rel_err(out.cpu().numpy(), ref, ref_abs) <= 1e-5
