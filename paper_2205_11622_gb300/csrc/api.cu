@@ -302,7 +302,11 @@ bool use_tc_fused(const slnr_opts* o, int32_t K, int32_t L, int64_t nnz) {
 //    (150k rows 64/32 295 | 110, 50k rows 100/48 148 | 71, 500k 64/64 588 |
 //    246), unless D widens the rows more than four times on a call of some
 //    size (uniform 220k rows 12/256 158 | 307);
-//  - fibers (<SpTTM,SpTTM>): D first (20M nonzeros 64/64 712 | 430, 1M 156 | 82);
+//  - fibers (<SpTTM,SpTTM>): D first (20M nonzeros 64/64 712 | 430, 1M 156 |
+//    82), unless D widens the rows more than twice and the tensor cores take a
+//    large call (2.5M 32/128 119 | 134);
+//  - sampled rows: row first where D widens them (R-MAT 718k rows 16/16/64
+//    825 | 1142, uniform 39k 16/16/128 40 | 48);
 //  - tensor cores: D first on graphs of fewer rows, where the row kernel's
 //    tiles of heavy rows set its time (50k rows 128/128 159 | 90, 220k 64/64
 //    201 | 128), row first on larger ones (500k 32/32 118 | 160, 1M 128/128
@@ -316,9 +320,10 @@ bool premul_first(const slnr_opts* o, PremulKind kind, int64_t nrows, int64_t nc
                   bool row_tc) {
   if (o->variant != SLNR_FUSED || nnz < 1 || nnz < ncols) return false;
   if (L > K && nnz > 64 * nrows) return false;  // long rows: the narrower rows are gathered
-  if (kind == kFibers) return true;
-  if (!row_tc) return L <= 4 * K || nnz < (int64_t(1) << 18);
   const int64_t k = 1024, few = (K <= 32 ? 128 : 256) * k;
+  if (kind == kFibers) return !row_tc || L <= 2 * K || nnz < 2048 * k;
+  if (kind == kSampledRows && L > 2 * K && nrows >= (L > 4 * K ? 0 : 64 * k)) return false;
+  if (!row_tc) return L <= 4 * K || nnz < 256 * k;
   if (L > 2 * K) return nrows < 64 * k;
   if (kind == kTwo) return nrows < few || nnz >= 8 * nrows;
   if (nrows >= few) return kind == kOne && K == 64 && L < 64 && nnz >= 8 * nrows;
@@ -393,7 +398,7 @@ Layout layout_mttkrp(const slnr_csf3* B, int32_t L, int variant) {
 }
 
 bool premul_spttm(const slnr_csf3* B, int32_t L, int32_t M, const slnr_opts* o) {
-  return premul_first(o, kFibers, B->nfibers, B->dim[2], B->nnz, L, M, false);
+  return premul_first(o, kFibers, B->nfibers, B->dim[2], B->nnz, L, M, use_tc_fused(o, L, M, B->nnz));
 }
 
 Layout layout_spttm_ttm(const slnr_csf3* B, int32_t L, int32_t M, const slnr_opts* o) {
