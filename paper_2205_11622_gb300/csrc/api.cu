@@ -131,6 +131,16 @@ struct Layout {
       if (total() <= budget || nw <= 1) return;
     }
   }
+  // windows of the fused MTTKRP kernels
+  size_t o_first2 = 0;
+  void mt_windows(int64_t nnz, int64_t nslices, int width) {
+    win = mt_window(nnz, nslices);
+    nw = (int)((nnz + win - 1) / win);
+    o_first = take(sizeof(int) * (size_t)nw);
+    o_first2 = take(sizeof(int) * (size_t)nw);
+    o_tail_row = take(sizeof(int) * (size_t)nw);
+    o_pieces = take(sizeof(float) * 2 * (size_t)nw * (size_t)width);
+  }
   size_t o_inter = 0, o_inter2 = 0;
   void inter(size_t bytes) { o_inter = take(bytes); }
   void inter2(size_t bytes) { o_inter2 = take(bytes); }
@@ -157,6 +167,12 @@ SplitPlan combine_plan(const SegPlan& g) {
 FlatPlan flat_plan(char* ws, const Layout& l) {
   return FlatPlan{reinterpret_cast<WsHeader*>(ws), l.win, l.nw, reinterpret_cast<int*>(ws + l.o_first),
                   reinterpret_cast<int*>(ws + l.o_tail_row), reinterpret_cast<float*>(ws + l.o_pieces)};
+}
+
+MtPlan mt_plan(char* ws, const Layout& l) {
+  return MtPlan{reinterpret_cast<WsHeader*>(ws), l.win, l.nw, reinterpret_cast<int*>(ws + l.o_first),
+                reinterpret_cast<int*>(ws + l.o_first2), reinterpret_cast<int*>(ws + l.o_tail_row),
+                reinterpret_cast<float*>(ws + l.o_pieces)};
 }
 
 UnitPlan unit_plan(char* ws, const Layout& l) {
@@ -389,8 +405,10 @@ slnr_status flat_sddmm_spmm(const CsrView& v, const float* C, const float* D, in
 
 Layout layout_mttkrp(const slnr_csf3* B, int32_t L, int variant) {
   Layout l;
-  l.units(B->nslices, B->nnz, L);
-  if (variant == SLNR_UNFUSED) {
+  if (variant == SLNR_FUSED) {
+    l.mt_windows(B->nnz, B->nslices, L);
+  } else {
+    l.units(B->nslices, B->nnz, L);
     l.split(B->nfibers, B->nnz, L);
     l.inter(sizeof(float) * (size_t)B->nfibers * (size_t)L);
   }
@@ -442,8 +460,11 @@ Layout layout_sddmm_spmm_gemm(const slnr_csr* B, int32_t K, int32_t L, int32_t M
 
 Layout layout_mttkrp_gemm(const slnr_csf3* B, int32_t L, int variant) {
   Layout l;
-  l.units(B->nslices, B->nnz, L);
-  if (variant == SLNR_UNFUSED) {
+  if (variant == SLNR_FUSED) {
+    l.mt_windows(B->nnz, B->nslices, L);
+    l.inter(sizeof(float) * (size_t)B->nslices * (size_t)L);      // the slices' rows
+  } else {
+    l.units(B->nslices, B->nnz, L);
     l.split(B->nfibers, B->nnz, L);
     l.inter(sizeof(float) * (size_t)B->nfibers * (size_t)L);      // per-fiber T
     l.inter2(sizeof(float) * (size_t)B->dim[0] * (size_t)L);      // the MTTKRP result
@@ -505,28 +526,33 @@ slnr_status wide_spmm_gemm(const CsrView& v, const float* C, const float* C2, in
   return SLNR_OK;
 }
 
-// MTTKRP (E NULL) or <MTTKRP,GEMM> (times E, L x M); the units are already listed
+// Fused MTTKRP (E NULL) or <MTTKRP,GEMM> (times E, L x M), any widths.
+slnr_status flat_mttkrp(const slnr_csf3* B, const float* C, const float* D, int32_t L, const float* E, int32_t M,
+                        float* A, char* ws, const Layout& l, cudaStream_t s) {
+  const MtPlan mp = mt_plan(ws, l);
+  float* U = E != nullptr ? reinterpret_cast<float*>(ws + l.o_inter) : nullptr;
+  SLNR_LAUNCH("mttkrp_first", launch_mt_first(*B, L, E != nullptr ? M : L, A, mp, s));
+  SLNR_LAUNCH("mttkrp", launch_mt(*B, C, D, L, U, A, mp, s));
+  if (E != nullptr && B->nnz > 0) SLNR_LAUNCH("slices_times", launch_slices_times(*B, L, M, U, E, A, s));
+  return SLNR_OK;
+}
+
+// Unfused MTTKRP (E NULL) or <MTTKRP,GEMM> (times E, L x M); the units are already listed
 slnr_status wide_mttkrp(const slnr_csf3* B, const float* C, const float* D, int32_t L, const float* E, int32_t M,
-                        float* A, char* ws, const Layout& l, const UnitPlan& up, int variant, bool tc,
-                        cudaStream_t s) {
-  if (variant == SLNR_FUSED) {
-    SLNR_LAUNCH("w_mttkrp_units", launch_w_mttkrp_units(L, *B, C, D, nullptr, up, s));
-    SLNR_LAUNCH("w_mttkrp_combine", launch_w_mttkrp_combine(L, *B, up, E, M, A, s));
-    return SLNR_OK;
-  }
+                        float* A, char* ws, const Layout& l, const UnitPlan& up, bool tc, cudaStream_t s) {
   const CsrView fv = fiber_view(B);
   const SplitPlan sp = split_plan(ws, l);
   float* T = reinterpret_cast<float*>(ws + l.o_inter);
   SLNR_LAUNCH("classify", launch_classify(fv, sp, s));
   SLNR_LAUNCH("w_spmm", launch_w_spmm(L, fv, D, nullptr, T, sp, s));
   SLNR_LAUNCH("w_combine", launch_w_combine(L, sp, nullptr, 0, T, s));
-  SLNR_LAUNCH("w_mttkrp_units", launch_w_mttkrp_units(L, *B, C, nullptr, T, up, s));
+  SLNR_LAUNCH("w_mttkrp_units", launch_w_mttkrp_units(L, *B, C, T, up, s));
   if (E == nullptr) {
-    SLNR_LAUNCH("w_mttkrp_combine", launch_w_mttkrp_combine(L, *B, up, nullptr, 0, A, s));
+    SLNR_LAUNCH("w_mttkrp_combine", launch_w_mttkrp_combine(L, *B, up, A, s));
     return SLNR_OK;
   }
   float* U = reinterpret_cast<float*>(ws + l.o_inter2);
-  SLNR_LAUNCH("w_mttkrp_combine", launch_w_mttkrp_combine(L, *B, up, nullptr, 0, U, s));
+  SLNR_LAUNCH("w_mttkrp_combine", launch_w_mttkrp_combine(L, *B, up, U, s));
   if (tc)
     SLNR_LAUNCH("tc_dense_gemm", launch_tc_dense_gemm(B->dim[0], L, M, U, E, A, sp.hdr, s));
   else
@@ -826,27 +852,28 @@ slnr_status slnr_mttkrp(const slnr_csf3* B, const float* C, const float* D, int3
   if (B->dim[0] == 0) return SLNR_OK;
   cudaStream_t s = static_cast<cudaStream_t>(opts->stream);
   char* ws = static_cast<char*>(opts->workspace);
+  const bool fused = opts->variant == SLNR_FUSED;
   SLNR_CHECK(begin(ws, s, opts->validate != 0,
-                   [&](WsHeader* h) { return launch_validate_csf(*B, h, s); }));
+                   [&](WsHeader* h) { return launch_validate_csf(*B, h, s); }, fused));
+  if (fused) {
+    SLNR_CHECK(flat_mttkrp(B, C, D, L, nullptr, 0, A, ws, l, s));
+    return finish(ws, s, opts->validate != 0);
+  }
   const UnitPlan up = unit_plan(ws, l);
   SLNR_LAUNCH("csf_units", launch_csf_units(*B, up, s));
   if (!pow2_dim(L)) {
-    SLNR_CHECK(wide_mttkrp(B, C, D, L, nullptr, 0, A, ws, l, up, opts->variant, false, s));
+    SLNR_CHECK(wide_mttkrp(B, C, D, L, nullptr, 0, A, ws, l, up, false, s));
     return finish(ws, s, opts->validate != 0);
   }
-  if (opts->variant == SLNR_FUSED) {
-    SLNR_LAUNCH("mttkrp_units", launch_mttkrp_units(L, *B, C, D, up, s));
-  } else {
-    const CsrView fv = fiber_view(B);
-    const SplitPlan sp = split_plan(ws, l);
-    float* T = reinterpret_cast<float*>(ws + l.o_inter);
-    SLNR_LAUNCH("classify", launch_classify(fv, sp, s));
-    SLNR_LAUNCH("spmm_chunks", launch_spmm_chunks(L, fv, D, sp, s));
-    SLNR_LAUNCH("spmm_rows", launch_spmm_rows(L, fv, D, T, s));
-    SLNR_LAUNCH("combine", launch_combine(L, sp, nullptr, 0, T, s));
-    SLNR_LAUNCH("mttkrp_stage2_units", launch_mttkrp_stage2_units(L, *B, T, C, up, s));
-  }
-  SLNR_LAUNCH("mttkrp_combine", launch_mttkrp_combine(L, *B, up, nullptr, 0, A, s));
+  const CsrView fv = fiber_view(B);
+  const SplitPlan sp = split_plan(ws, l);
+  float* T = reinterpret_cast<float*>(ws + l.o_inter);
+  SLNR_LAUNCH("classify", launch_classify(fv, sp, s));
+  SLNR_LAUNCH("spmm_chunks", launch_spmm_chunks(L, fv, D, sp, s));
+  SLNR_LAUNCH("spmm_rows", launch_spmm_rows(L, fv, D, T, s));
+  SLNR_LAUNCH("combine", launch_combine(L, sp, nullptr, 0, T, s));
+  SLNR_LAUNCH("mttkrp_stage2_units", launch_mttkrp_stage2_units(L, *B, T, C, up, s));
+  SLNR_LAUNCH("mttkrp_combine", launch_mttkrp_combine(L, *B, up, A, s));
   return finish(ws, s, opts->validate != 0);
 }
 
@@ -1009,15 +1036,17 @@ slnr_status slnr_mttkrp_gemm(const slnr_csf3* B, const float* C, const float* D,
   if (B->dim[0] == 0) return SLNR_OK;
   cudaStream_t s = static_cast<cudaStream_t>(opts->stream);
   char* ws = static_cast<char*>(opts->workspace);
+  const bool fused = opts->variant == SLNR_FUSED;
   SLNR_CHECK(begin(ws, s, opts->validate != 0,
-                   [&](WsHeader* h) { return launch_validate_csf(*B, h, s); }));
+                   [&](WsHeader* h) { return launch_validate_csf(*B, h, s); }, fused));
+  if (fused) {
+    SLNR_CHECK(flat_mttkrp(B, C, D, L, E, M, A, ws, l, s));
+    return finish(ws, s, opts->validate != 0);
+  }
   const UnitPlan up = unit_plan(ws, l);
   SLNR_LAUNCH("csf_units", launch_csf_units(*B, up, s));
   if (!all_pow2(L, M)) {
-    SLNR_CHECK(wide_mttkrp(B, C, D, L, E, M, A, ws, l, up, opts->variant, use_tc(opts, L, M), s));
-  } else if (opts->variant == SLNR_FUSED) {
-    SLNR_LAUNCH("mttkrp_units", launch_mttkrp_units(L, *B, C, D, up, s));
-    SLNR_LAUNCH("mttkrp_combine", launch_mttkrp_combine(L, *B, up, E, M, A, s));
+    SLNR_CHECK(wide_mttkrp(B, C, D, L, E, M, A, ws, l, up, use_tc(opts, L, M), s));
   } else {
     const CsrView fv = fiber_view(B);
     const SplitPlan sp = split_plan(ws, l);
@@ -1028,7 +1057,7 @@ slnr_status slnr_mttkrp_gemm(const slnr_csf3* B, const float* C, const float* D,
     SLNR_LAUNCH("spmm_rows", launch_spmm_rows(L, fv, D, T, s));
     SLNR_LAUNCH("combine", launch_combine(L, sp, nullptr, 0, T, s));
     SLNR_LAUNCH("mttkrp_stage2_units", launch_mttkrp_stage2_units(L, *B, T, C, up, s));
-    SLNR_LAUNCH("mttkrp_combine", launch_mttkrp_combine(L, *B, up, nullptr, 0, U, s));
+    SLNR_LAUNCH("mttkrp_combine", launch_mttkrp_combine(L, *B, up, U, s));
     if (use_tc(opts, L, M))
       SLNR_LAUNCH("tc_dense_gemm", launch_tc_dense_gemm(B->dim[0], L, M, U, E, A, sp.hdr, s));
     else

@@ -19,8 +19,8 @@ namespace slnr {
 // partials of a row in a fixed order (deterministic results).
 constexpr int kLightMax = 256;
 constexpr int kChunk = 256;
-// MTTKRP: a slice is cut into units of fibers that start within one window
-// of kUnitNnz nonzeros.
+// Unfused MTTKRP: a slice is cut into units of fibers that start within one
+// window of kUnitNnz nonzeros.
 constexpr int kUnitNnz = 512;
 // Tensor-core path: rows are cut into segments of at most kSegChunk nonzeros,
 // listed by length class (kSegClasses classes: (64,128], (32,64], ..., 2, 1,
@@ -38,8 +38,7 @@ struct WsHeader {        // first 256 bytes of every workspace
   int n_segs;            // segments of the tensor-core path
   int next_tile;         // tensor-core path: next item tile to hand to a CTA
   int next_row;          // fused <SDDMM,SpMM>: next block of rows to hand to a warp
-  int next_unit;         // fused MTTKRP: next unit to hand to a warp
-  int pad[56];
+  int pad[57];
 };
 static_assert(sizeof(WsHeader) == 256, "header is 256 bytes");
 
@@ -67,10 +66,6 @@ struct Unit {            // MTTKRP: window `u` of slice `slice`
   int u;
   int flo;               // fibers starting in the window: [flo, fhi)
   int fhi;
-  int p0;                // the window's nonzeros: [p0, p1)
-  int p1;
-  int ffirst;            // the fiber holding nonzero p0 (the last whose first nonzero is <= p0)
-  int pad;
 };
 
 // Validation flag bits

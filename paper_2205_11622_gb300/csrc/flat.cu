@@ -440,29 +440,15 @@ __global__ void __launch_bounds__(kCombineThreads) k_flat_combine(FlatArgs a) {
 
 bool aligned32(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0; }
 
-// A launch that may start while the kernel before it on the stream drains
-// (its grid_wait() waits for that kernel's results).
-template <typename K>
-cudaError_t launch_early(K k, int64_t grid, int threads, const FlatArgs& a, cudaStream_t s) {
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)SLNR_COUNTED(grid));
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.stream = s;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k, a);
-}
-
 template <int GS, int NCH, int MODE, int KIND>
 cudaError_t flat_launch(const FlatArgs& a, cudaStream_t s) {
   if (a.nw < 1) return cudaSuccess;
   cudaError_t e =
-      launch_early(k_flat<GS, NCH, MODE, KIND>, ceil_div(ceil_div(a.nw, 32 / GS), kFlatThreads / 32), kFlatThreads, a, s);
+      flat::launch_early(k_flat<GS, NCH, MODE, KIND>,
+                         SLNR_COUNTED(ceil_div(ceil_div(a.nw, 32 / GS), kFlatThreads / 32)), kFlatThreads, 0, s, a);
   if (e != cudaSuccess || a.nw < 2) return e;
-  return launch_early(k_flat_combine<GS, NCH, KIND>, ceil_div(a.nw, kCombineThreads), kCombineThreads, a, s);
+  return flat::launch_early(k_flat_combine<GS, NCH, KIND>, SLNR_COUNTED(ceil_div(a.nw, kCombineThreads)),
+                            kCombineThreads, 0, s, a);
 }
 
 template <int MODE, int KIND>

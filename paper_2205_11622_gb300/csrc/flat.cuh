@@ -8,6 +8,8 @@
 // stores.
 #pragma once
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace slnr {
@@ -198,6 +200,24 @@ struct Row {
     return f.x + f.y;
   }
 };
+
+// A launch that may start while the kernel before it on the stream drains
+// (its grid_wait() waits for that kernel's results).
+template <typename Args>
+cudaError_t launch_early(void (*kernel)(Args), int64_t grid, int threads, size_t smem, cudaStream_t s,
+                         const typename std::remove_cv<Args>::type& a) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, a);
+}
 
 }  // namespace flat
 }  // namespace slnr

@@ -70,6 +70,17 @@ struct FlatPlan {
   float* pieces;  // 2 x nw rows of the output width: heads, then tails
 };
 
+// Workspace pieces of the MTTKRP windows (mttkrp_flat.cu).
+struct MtPlan {
+  WsHeader* hdr;     // its flag word is zeroed by the call's first kernel
+  int win;           // nonzeros per window (mt_window)
+  int nw;            // windows: ceil(nnz / win)
+  int* first_slice;  // [nw]
+  int* first_fiber;  // [nw]
+  int* tail_slice;   // [nw]
+  float* pieces;     // 2 x nw rows of width L: heads, then tails
+};
+
 int device_sm_count();
 
 // Sets the calling thread's slnr_last_error() text (api.cu).
@@ -148,6 +159,10 @@ cudaError_t launch_flat_sampled(const CsrView& B, const float* C, const float* D
 cudaError_t launch_premul(int64_t M, int K, int L, const float* X, const float* X2, const float* D, float* G,
                           cudaStream_t s);
 
+// rows of A (width M) that slices with nonzeros own: U(s,:) . E into row crd1[s] (U nslices x L, E L x M)
+cudaError_t launch_slices_times(const slnr_csf3& B, int L, int M, const float* U, const float* E, float* A,
+                                cudaStream_t s);
+
 // sddmm.cu
 // fused <SDDMM,SpMM>: the heavy rows' chunks (partials) and the light rows in
 // one launch (plan.hdr->next_row must be 0: warps take work from it)
@@ -163,15 +178,19 @@ cudaError_t launch_sddmm_rows(const CsrView& B, const float* C, const float* D, 
 cudaError_t launch_sddmm_chunks(const CsrView& B, const float* C, const float* D, int L, float* Y,
                                 const SplitPlan& plan, cudaStream_t s);
 
-// mttkrp.cu
-cudaError_t launch_mttkrp_units(int L, const slnr_csf3& B, const float* C, const float* D,
-                                const UnitPlan& plan, cudaStream_t s);
+// mttkrp_flat.cu -- fused MTTKRP, any widths, in two steps of a call: the windows' first slices and fibers (and the rows of A
+// without nonzeros, zero), then the sums
+int mt_window(int64_t nnz, int64_t nslices);
+// (M: width of A; with U, nslices x L, not NULL the slices' rows go to U instead of A)
+cudaError_t launch_mt_first(const slnr_csf3& B, int L, int M, float* A, const MtPlan& plan, cudaStream_t s);
+cudaError_t launch_mt(const slnr_csf3& B, const float* C, const float* D, int L, float* U, float* A,
+                      const MtPlan& plan, cudaStream_t s);
+
+// mttkrp.cu -- the unfused variants
 cudaError_t launch_mttkrp_stage2_units(int L, const slnr_csf3& B, const float* T, const float* C,
                                        const UnitPlan& plan, cudaStream_t s);
-// A(i,:) = sum of slice i's unit partials (width L); with E (L x M) not NULL,
-// that sum times E (A has width M).
-cudaError_t launch_mttkrp_combine(int L, const slnr_csf3& B, const UnitPlan& plan, const float* E, int M,
-                                  float* A, cudaStream_t s);
+// A(i,:) = sum of slice i's unit partials (width L)
+cudaError_t launch_mttkrp_combine(int L, const slnr_csf3& B, const UnitPlan& plan, float* A, cudaStream_t s);
 
 // api.cu -- the size that a heavy-row split of B takes (what the built-in scratch is measured by), and
 // slnr_sddmm_spmm (fused) with windows long enough to fit opts->workspace_bytes
@@ -199,11 +218,10 @@ cudaError_t launch_w_sddmm_spmm(const CsrView& B, const float* C, const float* D
                                 float* A, float* Y, const SplitPlan& plan, cudaStream_t s);
 cudaError_t launch_w_sddmm_spmm_gemm_tiles(const CsrView& B, const float* C, const float* D, int K, const float* F,
                                            int L, const float* W, int M, float* A, cudaStream_t s);
-// MTTKRP unit partials: fused (T == NULL) or from the per-fiber T (unfused)
-cudaError_t launch_w_mttkrp_units(int L, const slnr_csf3& B, const float* C, const float* D, const float* T,
-                                  const UnitPlan& plan, cudaStream_t s);
-cudaError_t launch_w_mttkrp_combine(int L, const slnr_csf3& B, const UnitPlan& plan, const float* E, int M, float* A,
-                                    cudaStream_t s);
+// unfused MTTKRP: unit partials from the per-fiber T
+cudaError_t launch_w_mttkrp_units(int L, const slnr_csf3& B, const float* C, const float* T, const UnitPlan& plan,
+                                  cudaStream_t s);
+cudaError_t launch_w_mttkrp_combine(int L, const slnr_csf3& B, const UnitPlan& plan, float* A, cudaStream_t s);
 
 // peaks.cu -- peaks measured by the library's own kernels (TFLOP/s, GB/s)
 cudaError_t peak_ffma(cudaStream_t s, double* tflops);

@@ -21,10 +21,17 @@ constexpr int kPmRows = 128;
 constexpr int kPmK = 32;
 constexpr int kPmPitch = kPmRows + 4;  // keeps 16-byte alignment and spreads the transposed stores
 
-template <int BN, bool H>
+// kSlices: row r of X belongs to slice r of a CSF tensor and goes to row crd1[r]
+// of G, unless the slice has no nonzeros.
+enum PremulRows { kPlain = 0, kHadamard = 1, kSlices = 2 };
+
+template <int BN, int ROWS>
 __global__ void __launch_bounds__(kPmThreads) k_premul(int64_t M, int K, int L, const float* __restrict__ X,
                                                        const float* __restrict__ X2, const float* __restrict__ D,
-                                                       float* __restrict__ G) {
+                                                       float* __restrict__ G, const int32_t* __restrict__ crd1,
+                                                       const int32_t* __restrict__ pos2,
+                                                       const int32_t* __restrict__ pos3) {
+  constexpr bool H = ROWS == kHadamard;
   constexpr int CG = BN / 4;                  // threads along the columns
   constexpr int RG = kPmThreads / CG;         // threads along the rows
   constexpr int RPT = kPmRows / RG;           // rows per thread
@@ -83,30 +90,50 @@ __global__ void __launch_bounds__(kPmThreads) k_premul(int64_t M, int K, int L, 
     const float2 a = flat::unpack2(acc[i][0]), b = flat::unpack2(acc[i][1]), c = flat::unpack2(acc[i][2]),
                  d = flat::unpack2(acc[i][3]);
     const int64_t r = r0 + rg * RPT + 2 * i;
-    if (r < M) reinterpret_cast<float4*>(G + r * L + c0)[cg] = make_float4(a.x, b.x, c.x, d.x);
-    if (r + 1 < M) reinterpret_cast<float4*>(G + (r + 1) * L + c0)[cg] = make_float4(a.y, b.y, c.y, d.y);
+    auto put = [&](int64_t row, float4 v) {
+      if (row >= M) return;
+      if constexpr (ROWS == kSlices) {
+        if (__ldg(pos3 + __ldg(pos2 + row)) == __ldg(pos3 + __ldg(pos2 + row + 1))) return;
+        row = __ldg(crd1 + row);
+      }
+      reinterpret_cast<float4*>(G + row * L + c0)[cg] = v;
+    };
+    put(r, make_float4(a.x, b.x, c.x, d.x));
+    put(r + 1, make_float4(a.y, b.y, c.y, d.y));
   }
 }
 
 template <int BN>
 cudaError_t premul_launch(int64_t M, int K, int L, const float* X, const float* X2, const float* D, float* G,
-                          cudaStream_t s) {
+                          const slnr_csf3* B, cudaStream_t s) {
   const dim3 grid((unsigned)SLNR_COUNTED(ceil_div(M, kPmRows)), (unsigned)ceil_div(L, BN));
-  if (X2 == nullptr)
-    k_premul<BN, false><<<grid, kPmThreads, 0, s>>>(M, K, L, X, nullptr, D, G);
+  if (B != nullptr)
+    k_premul<BN, kSlices><<<grid, kPmThreads, 0, s>>>(M, K, L, X, nullptr, D, G, B->crd1, B->pos2, B->pos3);
+  else if (X2 != nullptr)
+    k_premul<BN, kHadamard><<<grid, kPmThreads, 0, s>>>(M, K, L, X, X2, D, G, nullptr, nullptr, nullptr);
   else
-    k_premul<BN, true><<<grid, kPmThreads, 0, s>>>(M, K, L, X, X2, D, G);
+    k_premul<BN, kPlain><<<grid, kPmThreads, 0, s>>>(M, K, L, X, nullptr, D, G, nullptr, nullptr, nullptr);
   return cudaGetLastError();
+}
+
+cudaError_t premul_width(int64_t M, int K, int L, const float* X, const float* X2, const float* D, float* G,
+                         const slnr_csf3* B, cudaStream_t s) {
+  if (M <= 0) return cudaSuccess;
+  if (L <= 16) return premul_launch<16>(M, K, L, X, X2, D, G, B, s);
+  if (L <= 32) return premul_launch<32>(M, K, L, X, X2, D, G, B, s);
+  return premul_launch<64>(M, K, L, X, X2, D, G, B, s);
 }
 
 }  // namespace
 
 cudaError_t launch_premul(int64_t M, int K, int L, const float* X, const float* X2, const float* D, float* G,
                           cudaStream_t s) {
-  if (M <= 0) return cudaSuccess;
-  if (L <= 16) return premul_launch<16>(M, K, L, X, X2, D, G, s);
-  if (L <= 32) return premul_launch<32>(M, K, L, X, X2, D, G, s);
-  return premul_launch<64>(M, K, L, X, X2, D, G, s);
+  return premul_width(M, K, L, X, X2, D, G, nullptr, s);
+}
+
+cudaError_t launch_slices_times(const slnr_csf3& B, int L, int M, const float* U, const float* E, float* A,
+                                cudaStream_t s) {
+  return premul_width(B.nslices, L, M, U, nullptr, E, A, &B, s);
 }
 
 }  // namespace slnr

@@ -426,19 +426,14 @@ __global__ void __launch_bounds__(kWThreads) k_w_sddmm_spmm_gemm_tiles(int nrows
   wtile_times_d(T, L, Wm, M, Ds, A, r0, nrows, keep);
 }
 
-// MTTKRP over units (the fibers of a slice that start in one window of
-// kUnitNnz nonzeros): a warp per unit, its fibers in order; per fiber the
-// producer T(l) = sum_k B(i,j,k) D(k,l) (or, unfused, T's row read from
-// memory) and the consumer acc += T .* C(j,:); one partial row per unit.
-template <int NCH, bool TG>
+// Unfused MTTKRP over units (the fibers of a slice that start in one window of
+// kUnitNnz nonzeros): a warp per unit, its fibers in order; acc += T .* C(j,:)
+// with T's row read from memory; one partial row per unit.
+template <int NCH>
 __global__ void __launch_bounds__(kWThreads) k_w_mttkrp_units(const WsHeader* __restrict__ hdr,
                                                               const Unit* __restrict__ units, int max_units,
                                                               const int32_t* __restrict__ crd2,
-                                                              const int32_t* __restrict__ pos3,
-                                                              const int32_t* __restrict__ crd3,
-                                                              const float* __restrict__ vals,
                                                               const float* __restrict__ C,
-                                                              const float* __restrict__ D,
                                                               const float* __restrict__ Tg, int L,
                                                               float* __restrict__ partial) {
   const int lane = threadIdx.x & 31;
@@ -451,10 +446,7 @@ __global__ void __launch_bounds__(kWThreads) k_w_mttkrp_units(const WsHeader* __
     for (int f = un.flo; f < un.fhi; ++f) {
       const int j = __ldg(crd2 + f);
       float4 t[NCH], c[NCH];
-      if constexpr (TG)
-        wload(t, Tg + (int64_t)f * L, L, lane);
-      else
-        wgather<NCH, false>(t, crd3, vals, __ldg(pos3 + f), __ldg(pos3 + f + 1), D, nullptr, L, lane);
+      wload(t, Tg + (int64_t)f * L, L, lane);
       wload(c, C + (int64_t)j * L, L, lane);
 #pragma unroll
       for (int i = 0; i < NCH; ++i) {
@@ -469,17 +461,13 @@ __global__ void __launch_bounds__(kWThreads) k_w_mttkrp_units(const WsHeader* __
 }
 
 // A(i,:) = the sum of slice i's unit partials (width L), a warp per slice,
-// units in order; with E (L x M) the sum is staged in shared memory and
-// A(i,:) = sum . E (width M).  Rows of A without a slice are zeroed before.
+// units in order.  Rows of A without a slice are zeroed before.
 template <int NCH>
 __global__ void __launch_bounds__(kWThreads) k_w_mttkrp_combine(int nslices, const int32_t* __restrict__ crd1,
                                                                 const SliceUnits* __restrict__ sus,
                                                                 const float* __restrict__ partial, int L,
-                                                                const float* __restrict__ E, int M,
                                                                 float* __restrict__ A) {
-  extern __shared__ float4 wsm4[];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  float* u = reinterpret_cast<float*>(wsm4) + (size_t)wib * L;
+  const int lane = threadIdx.x & 31;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < nslices; q += nwarps) {
     const SliceUnits su = sus[q];
@@ -497,20 +485,7 @@ __global__ void __launch_bounds__(kWThreads) k_w_mttkrp_combine(int nslices, con
         s[h].w += x[h].w;
       }
     }
-    if (E == nullptr) {
-      wstore(A + (int64_t)i * L, s, L, lane);
-      continue;
-    }
-    __syncwarp();
-#pragma unroll
-    for (int h = 0; h < NCH; ++h)
-      if (4 * (lane + 32 * h) < L) reinterpret_cast<float4*>(u)[lane + 32 * h] = s[h];
-    __syncwarp();
-    for (int m4 = lane; 4 * m4 < M; m4 += 32) {
-      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int l = 0; l < L; ++l) fma4(a, u[l], __ldg(reinterpret_cast<const float4*>(E + (int64_t)l * M) + m4));
-      reinterpret_cast<float4*>(A + (int64_t)i * M)[m4] = a;
-    }
+    wstore(A + (int64_t)i * L, s, L, lane);
   }
 }
 
@@ -629,32 +604,23 @@ cudaError_t launch_w_sddmm_spmm_gemm_tiles(const CsrView& B, const float* C, con
   return cudaGetLastError();
 }
 
-cudaError_t launch_w_mttkrp_units(int L, const slnr_csf3& B, const float* C, const float* D, const float* T,
-                                  const UnitPlan& plan, cudaStream_t s) {
+cudaError_t launch_w_mttkrp_units(int L, const slnr_csf3& B, const float* C, const float* T, const UnitPlan& plan,
+                                  cudaStream_t s) {
   if (plan.max_units <= 0 || B.nslices <= 0) return cudaSuccess;
-  const unsigned grid = w_grid(plan.max_units);
   SLNR_NCH_SWITCH(L, NC, {
-    if (T == nullptr)
-      k_w_mttkrp_units<NC, false><<<SLNR_COUNTED(grid), kWThreads, 0, s>>>(plan.hdr, plan.units, plan.max_units, B.crd2, B.pos3,
-                                                             B.crd3, B.vals, C, D, nullptr, L, plan.partial);
-    else
-      k_w_mttkrp_units<NC, true><<<SLNR_COUNTED(grid), kWThreads, 0, s>>>(plan.hdr, plan.units, plan.max_units, B.crd2, B.pos3,
-                                                            B.crd3, B.vals, C, D, T, L, plan.partial);
+    k_w_mttkrp_units<NC><<<SLNR_COUNTED(w_grid(plan.max_units)), kWThreads, 0, s>>>(plan.hdr, plan.units, plan.max_units,
+                                                                                   B.crd2, C, T, L, plan.partial);
   });
   return cudaGetLastError();
 }
 
-cudaError_t launch_w_mttkrp_combine(int L, const slnr_csf3& B, const UnitPlan& plan, const float* E, int M, float* A,
-                                    cudaStream_t s) {
+cudaError_t launch_w_mttkrp_combine(int L, const slnr_csf3& B, const UnitPlan& plan, float* A, cudaStream_t s) {
   if (B.dim[0] <= 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(A, 0, sizeof(float) * (size_t)B.dim[0] * (size_t)(E != nullptr ? M : L), s);
+  const cudaError_t e = cudaMemsetAsync(A, 0, sizeof(float) * (size_t)B.dim[0] * (size_t)L, s);
   if (e != cudaSuccess || B.nslices <= 0) return e;
-  const size_t smem = E != nullptr ? sizeof(float) * (kWThreads / 32) * (size_t)L : 0;
   SLNR_NCH_SWITCH(L, NC, {
-    e = w_smem(k_w_mttkrp_combine<NC>, smem);
-    if (e != cudaSuccess) return e;
-    k_w_mttkrp_combine<NC><<<SLNR_COUNTED(w_grid(B.nslices)), kWThreads, smem, s>>>(B.nslices, B.crd1, plan.slice_units,
-                                                                        plan.partial, L, E, M, A);
+    k_w_mttkrp_combine<NC><<<SLNR_COUNTED(w_grid(B.nslices)), kWThreads, 0, s>>>(B.nslices, B.crd1, plan.slice_units,
+                                                                               plan.partial, L, A);
   });
   return cudaGetLastError();
 }

@@ -136,3 +136,50 @@ def test_split_product_error(slnr, K, L, two):
     dB, dd = P.to_device(w)
     out = slnr.run(w.op, dB, dd, allow_tf32=True)
     assert P.rel_err(out.cpu().numpy(), ref, ref_abs) <= 1e-5
+
+
+def csf(kind, rng, d1, d2, seed):
+    """CSF tensors whose slices and fibers end at window edges, span many windows, or are empty in runs."""
+    if kind == "few":            # fewer nonzeros than a window
+        shape = [[1, 2], [], [3]]
+    elif kind == "long":         # one slice over hundreds of windows, single-nonzero slices around it
+        shape = [[1]] * 20 + [list(rng.integers(1, 90, 700))] + [[1, 1]] * 9 + [[64] * 16] + [[32], [32], [64]]
+    elif kind == "empty_runs":   # runs of empty slices and of empty fibers, shorter and longer than a step
+        shape = []
+        for n in (1, 7, 9, 40):
+            shape += [[5, 1] + [0] * n + [2]] + [[]] * n
+        shape += [[0] * 70 + [3] + [0] * 33, [40]] + [[0, 0]] * 12
+    pos2, pos3, crd2, crd3 = [0], [0], [], []
+    for s in shape:
+        crd2 += sorted(rng.choice(d1, len(s), replace=False).tolist())
+        for n in s:
+            crd3 += sorted(rng.choice(d2, int(n), replace=False).tolist())
+            pos3.append(len(crd3))
+        pos2.append(len(crd2))
+    d0 = 2 * len(shape) + 5
+    crd1 = np.sort(rng.choice(d0, len(shape), replace=False))
+    a = lambda x: np.asarray(x, np.int32)  # noqa: E731
+    return wl.CSF3((d0, d1, d2), a([0, len(shape)]), a(crd1), a(pos2), a(crd2), a(pos3), a(crd3),
+                   wl.uniform(wl.Rng(seed), len(crd3), -1, 1))
+
+
+@pytest.mark.parametrize("L,M", [(4, 8), (8, 4), (12, 36), (16, 16), (32, 64), (48, 100), (64, 32), (128, 260), (256, 16),
+                                 (260, 20), (512, 64), (1024, 12)])
+@pytest.mark.parametrize("kind", ["few", "long", "empty_runs"])
+def test_mttkrp_windows(slnr, L, M, kind):
+    rng = np.random.default_rng(L + M)
+    d1, d2 = 900, 120
+    B = csf(kind, rng, d1, d2, 0x51A4 + L)
+    r = wl.Rng(0x51A4 + M)
+    C, D, E = wl.uniform(r, (d1, L), -1, 1), wl.uniform(r, (d2, L), -1, 1), wl.uniform(r, (L, M), -1, 1)
+    for op, dense, dims in (("mttkrp", {"C": C, "D": D}, {"L": L}), ("mttkrp_gemm", {"C": C, "D": D, "E": E}, {"L": L, "M": M})):
+        w = wl.Workload(kind, op, B, dense, dims)
+        ref, ref_abs = oracle.get().run(w)
+        dB, dd = P.to_device(w)
+        for aligned in (True, False):
+            out = torch.full((B.dims[0], M if op == "mttkrp_gemm" else L), float("nan"), device="cuda")
+            if not aligned:
+                out, dd = shifted(out), {k: shifted(v) for k, v in dd.items()}
+            slnr.run(op, dB, dd, out=out)
+            assert slnr.device_flags() == 0
+            assert P.rel_err(out.cpu().numpy(), ref, ref_abs) <= P.TOL_FP32
