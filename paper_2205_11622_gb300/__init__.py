@@ -309,23 +309,48 @@ def device_flags(workspace=None) -> int:
     return int(buf[12:16].view(_torch().int32).item())
 
 
-def _opts(variant, allow_tf32, validate, stream):
-    torch = _torch()
-    v = {"fused": FUSED, "unfused": UNFUSED}.get(variant, variant)
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return slnr_opts(int(v), int(bool(allow_tf32)), int(bool(validate)), 0, ctypes.c_void_p(s.cuda_stream), None, 0)
+_VARIANTS = {"fused": FUSED, "unfused": UNFUSED, FUSED: FUSED, UNFUSED: UNFUSED}
+_ERR_WORKSPACE = 4
 
 
-def _attach_ws(opts, nbytes, workspace):
-    torch = _torch()
+def _stream_ptr(stream) -> int:
+    """The cudaStream_t of a torch stream (None: the current device's current stream)."""
+    if stream is not None:
+        return stream.cuda_stream
+    c = _torch()._C
+    return c._cuda_getCurrentRawStream(c._cuda_getDevice())
+
+
+def _run(name, B, args, sizes, variant, allow_tf32, validate, workspace, stream):
+    """Call entry point `name` with the structure B, `args` and the options.
+
+    The workspace that is there is tried first: the library checks its size
+    before it enqueues anything and says SLNR_ERR_WORKSPACE if it is too small;
+    only then is the size asked for (with `sizes`) and the buffer grown.  Small
+    calls are bound by this function, not by their kernels.
+    """
+    L = _lib if _lib is not None else lib()
+    s = _stream_ptr(stream)
     if workspace is None:
-        dev = torch.cuda.current_device()
-        workspace = _default_ws.setdefault((dev, opts.stream), Workspace(device=f"cuda:{dev}"))
-    buf = workspace.get(nbytes)
+        dev = _torch()._C._cuda_getDevice()
+        workspace = _default_ws.get((dev, s))
+        if workspace is None:
+            workspace = _default_ws.setdefault((dev, s), Workspace(device=f"cuda:{dev}"))
+    v = _VARIANTS.get(variant)
+    o = slnr_opts(int(variant) if v is None else v, 1 if allow_tf32 else 0, 1 if validate else 0, 0, s, None, 0)
+    bs, os_ = ctypes.byref(B), ctypes.byref(o)
+    status = _ERR_WORKSPACE
+    buf = workspace.buf
+    if buf is not None:
+        o.workspace, o.workspace_bytes = buf.data_ptr(), buf.numel()
+        status = getattr(L, name)(bs, *args, os_)
+    if status == _ERR_WORKSPACE:
+        buf = workspace.get(_query(name + "_workspace", bs, *sizes, os_))
+        o.workspace, o.workspace_bytes = buf.data_ptr(), buf.numel()
+        status = getattr(L, name)(bs, *args, os_)
     _last_ws[0] = buf
-    opts.workspace = buf.data_ptr()
-    opts.workspace_bytes = buf.numel()
-    return buf
+    if status != 0:
+        raise SlnrError(status, name, last_error())
 
 
 def _dense(x, name):
@@ -343,11 +368,9 @@ def spmm_gemm(B: DeviceCSR, C, D, out=None, variant="fused", allow_tf32=True, va
     K, L = C.shape[1], D.shape[1]
     if out is None:
         out = torch.empty((B.nrows, L), dtype=torch.float32, device=C.device)
-    o = _opts(variant, allow_tf32, validate, stream)
-    bs = B.c_struct()
-    n = _query("slnr_spmm_gemm_workspace", ctypes.byref(bs), K, L, ctypes.byref(o))
-    _keep = _attach_ws(o, n, workspace)
-    _check(slnr_spmm_gemm(bs, C.data_ptr(), K, D.data_ptr(), L, out.data_ptr(), o), "slnr_spmm_gemm")
+    _run("slnr_spmm_gemm", B.c_struct(),
+         (C.data_ptr(), K, D.data_ptr(), L, out.data_ptr()),
+         (K, L), variant, allow_tf32, validate, workspace, stream)
     return out
 
 
@@ -374,12 +397,9 @@ def sddmm_spmm(B: DeviceCSR, C, D, E, out=None, variant="fused", allow_tf32=True
     L, K = C.shape[1], E.shape[1]
     if out is None:
         out = torch.empty((B.nrows, K), dtype=torch.float32, device=C.device)
-    o = _opts(variant, allow_tf32, validate, stream)
-    bs = B.c_struct()
-    n = _query("slnr_sddmm_spmm_workspace", ctypes.byref(bs), L, K, ctypes.byref(o))
-    _keep = _attach_ws(o, n, workspace)
-    _check(slnr_sddmm_spmm(bs, C.data_ptr(), D.data_ptr(), L, E.data_ptr(), K, out.data_ptr(), o),
-           "slnr_sddmm_spmm")
+    _run("slnr_sddmm_spmm", B.c_struct(),
+         (C.data_ptr(), D.data_ptr(), L, E.data_ptr(), K, out.data_ptr()),
+         (L, K), variant, allow_tf32, validate, workspace, stream)
     return out
 
 
@@ -391,11 +411,9 @@ def mttkrp(B: DeviceCSF3, C, D, out=None, variant="fused", allow_tf32=True, vali
     L = C.shape[1]
     if out is None:
         out = torch.empty((B.dims[0], L), dtype=torch.float32, device=C.device)
-    o = _opts(variant, allow_tf32, validate, stream)
-    bs = B.c_struct()
-    n = _query("slnr_mttkrp_workspace", ctypes.byref(bs), L, ctypes.byref(o))
-    _keep = _attach_ws(o, n, workspace)
-    _check(slnr_mttkrp(bs, C.data_ptr(), D.data_ptr(), L, out.data_ptr(), o), "slnr_mttkrp")
+    _run("slnr_mttkrp", B.c_struct(),
+         (C.data_ptr(), D.data_ptr(), L, out.data_ptr()),
+         (L,), variant, allow_tf32, validate, workspace, stream)
     return out
 
 
@@ -414,13 +432,11 @@ def spttm_ttm(B: DeviceCSF3, C, D, out=None, variant="fused", allow_tf32=True, v
         out = (torch.empty(2, dtype=i32, device=dev), torch.empty(max(B.nslices, 1), dtype=i32, device=dev),
                torch.empty(B.nslices + 1, dtype=i32, device=dev), torch.empty(max(B.nfibers, 1), dtype=i32, device=dev),
                torch.empty((B.nfibers, M), dtype=torch.float32, device=dev))
-    o = _opts(variant, allow_tf32, validate, stream)
-    bs = B.c_struct()
-    n = _query("slnr_spttm_ttm_workspace", ctypes.byref(bs), L, M, ctypes.byref(o))
-    _keep = _attach_ws(o, n, workspace)
     p1, c1, p2, c2, v = out
-    _check(slnr_spttm_ttm(bs, C.data_ptr(), L, D.data_ptr(), M, p1.data_ptr(), c1.data_ptr(), p2.data_ptr(),
-                          c2.data_ptr(), v.data_ptr(), o), "slnr_spttm_ttm")
+    _run("slnr_spttm_ttm", B.c_struct(),
+         (C.data_ptr(), L, D.data_ptr(), M, p1.data_ptr(), c1.data_ptr(),
+          p2.data_ptr(), c2.data_ptr(), v.data_ptr()),
+         (L, M), variant, allow_tf32, validate, workspace, stream)
     return p1, c1[:B.nslices], p2, c2[:B.nfibers], v
 
 
@@ -432,12 +448,9 @@ def sddmm_spmm_gemm(B: DeviceCSR, C, D, F, W, out=None, variant="fused", allow_t
     K, L, M = C.shape[1], F.shape[1], W.shape[1]
     if out is None:
         out = torch.empty((B.nrows, M), dtype=torch.float32, device=C.device)
-    o = _opts(variant, allow_tf32, validate, stream)
-    bs = B.c_struct()
-    n = _query("slnr_sddmm_spmm_gemm_workspace", ctypes.byref(bs), K, L, M, ctypes.byref(o))
-    _keep = _attach_ws(o, n, workspace)
-    _check(slnr_sddmm_spmm_gemm(bs, C.data_ptr(), D.data_ptr(), K, F.data_ptr(), L, W.data_ptr(), M,
-                                out.data_ptr(), o), "slnr_sddmm_spmm_gemm")
+    _run("slnr_sddmm_spmm_gemm", B.c_struct(),
+         (C.data_ptr(), D.data_ptr(), K, F.data_ptr(), L, W.data_ptr(), M, out.data_ptr()),
+         (K, L, M), variant, allow_tf32, validate, workspace, stream)
     return out
 
 
@@ -449,12 +462,9 @@ def mttkrp_gemm(B: DeviceCSF3, C, D, E, out=None, variant="fused", allow_tf32=Tr
     L, M = C.shape[1], E.shape[1]
     if out is None:
         out = torch.empty((B.dims[0], M), dtype=torch.float32, device=C.device)
-    o = _opts(variant, allow_tf32, validate, stream)
-    bs = B.c_struct()
-    n = _query("slnr_mttkrp_gemm_workspace", ctypes.byref(bs), L, M, ctypes.byref(o))
-    _keep = _attach_ws(o, n, workspace)
-    _check(slnr_mttkrp_gemm(bs, C.data_ptr(), D.data_ptr(), L, E.data_ptr(), M, out.data_ptr(), o),
-           "slnr_mttkrp_gemm")
+    _run("slnr_mttkrp_gemm", B.c_struct(),
+         (C.data_ptr(), D.data_ptr(), L, E.data_ptr(), M, out.data_ptr()),
+         (L, M), variant, allow_tf32, validate, workspace, stream)
     return out
 
 
@@ -466,12 +476,9 @@ def spmmh_gemm(B: DeviceCSR, C, D, E, out=None, variant="fused", allow_tf32=True
     J, L = C.shape[1], E.shape[1]
     if out is None:
         out = torch.empty((B.nrows, L), dtype=torch.float32, device=C.device)
-    o = _opts(variant, allow_tf32, validate, stream)
-    bs = B.c_struct()
-    n = _query("slnr_spmmh_gemm_workspace", ctypes.byref(bs), J, L, ctypes.byref(o))
-    _keep = _attach_ws(o, n, workspace)
-    _check(slnr_spmmh_gemm(bs, C.data_ptr(), D.data_ptr(), J, E.data_ptr(), L, out.data_ptr(), o),
-           "slnr_spmmh_gemm")
+    _run("slnr_spmmh_gemm", B.c_struct(),
+         (C.data_ptr(), D.data_ptr(), J, E.data_ptr(), L, out.data_ptr()),
+         (J, L), variant, allow_tf32, validate, workspace, stream)
     return out
 
 
