@@ -129,8 +129,8 @@ cudaError_t launch_tc_spmm_gemm(int K, int L, const CsrView& B, const float* C, 
                                 const SegPlan& plan, cudaStream_t s, const float* C2 = nullptr);
 cudaError_t launch_tc_dense_gemm(int64_t M, int K, int L, const float* T, const float* D, float* A,
                                  WsHeader* hdr, cudaStream_t s);
-// G = X . D, or (X .* X2) . D (X, X2: M x K, D: K x L): X in two tf32 parts,
-// D rounded to tf32 (hdr zeroed by the call: the kernel takes tiles from it)
+// tc_premul.cu -- G = X . D, or (X .* X2) . D (X, X2: M x K, D: K x L): X in two
+// tf32 parts, D rounded to tf32 (hdr: its flag word takes a timeout)
 bool tc_split_supported(int K, int L);
 cudaError_t launch_tc_premul(int64_t M, int K, int L, const float* X, const float* X2, const float* D, float* G,
                              WsHeader* hdr, cudaStream_t s);

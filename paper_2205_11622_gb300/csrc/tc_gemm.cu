@@ -253,13 +253,7 @@ __device__ __forceinline__ int mbar_wait_or_end(uint64_t* bar, uint32_t parity, 
 // X[k,:] .* X2[k,:] (<SpMMH,GEMM>); kDense: rows of a materialised T.
 // kSampled (<SDDMM,SpMM,GEMM>): the row of stored (i,j) is F(j,:) scaled by
 // the sampled product B(i,j) <C(i,:), D(j,:)>.
-// kSplit, kSplitH: dense rows of X, or of X .* X2, each value split into the
-// sum of two tf32 values (hi, and lo = x - hi rounded), so that only D's
-// rounding is left in the product.
-enum TcMode { kSegments = 0, kDense = 1, kSegmentsH = 2, kSampled = 3, kSplit = 4, kSplitH = 5 };
-__host__ __device__ constexpr bool tc_dense_mode(int mode) { return mode == kDense || mode == kSplit || mode == kSplitH; }
-// tf32 values per value of a T row
-__host__ __device__ constexpr int tc_parts(int mode) { return mode == kSplit || mode == kSplitH ? 2 : 1; }
+enum TcMode { kSegments = 0, kDense = 1, kSegmentsH = 2, kSampled = 3 };
 
 // Columns of the T tile and of D^T: K, padded to one 128-byte swizzle atom
 // (32 tf32 values) when K = 16; the padding columns hold zeros.
@@ -267,12 +261,10 @@ __host__ __device__ constexpr int tc_kt(int K) { return K < 32 ? 32 : K; }
 
 // Number of T / accumulator buffers: up to four, as many as fit beside D^T
 // in shared memory (200 KB budget) and in tensor memory (512 columns).
-// P parts of every T value lie in one tile of P KT columns (the lo parts after
-// the hi parts).
-__host__ __device__ constexpr int tc_nbuf(int K, int L, int P) {
-  return ((size_t)4 * kTcRows * P * tc_kt(K) * 4 + (size_t)L * tc_kt(K) * 4 + 1024 <= (size_t)200 * 1024 && 4 * L <= 512)
+__host__ __device__ constexpr int tc_nbuf(int K, int L) {
+  return ((size_t)4 * kTcRows * tc_kt(K) * 4 + (size_t)L * tc_kt(K) * 4 + 1024 <= (size_t)200 * 1024 && 4 * L <= 512)
              ? 4
-             : ((size_t)2 * kTcRows * P * tc_kt(K) * 4 + (size_t)L * tc_kt(K) * 4 + 1024 <= (size_t)200 * 1024 &&
+             : ((size_t)2 * kTcRows * tc_kt(K) * 4 + (size_t)L * tc_kt(K) * 4 + 1024 <= (size_t)200 * 1024 &&
                 2 * L <= 512)
                    ? 2
                    : 1;
@@ -280,8 +272,8 @@ __host__ __device__ constexpr int tc_nbuf(int K, int L, int P) {
 
 // Tensor memory columns a CTA allocates: its NBUF accumulators (L columns
 // each), at least the 32 columns an allocation takes.
-__host__ __device__ constexpr uint32_t tc_tmem_cols(int K, int L, int P) {
-  return tc_nbuf(K, L, P) * L < 32 ? 32u : (uint32_t)(tc_nbuf(K, L, P) * L);
+__host__ __device__ constexpr uint32_t tc_tmem_cols(int K, int L) {
+  return tc_nbuf(K, L) * L < 32 ? 32u : (uint32_t)(tc_nbuf(K, L) * L);
 }
 
 // Epilogue staging: each of the four epilogue warps stages its 32 rows, one
@@ -294,17 +286,17 @@ __host__ __device__ constexpr uint32_t tc_tmem_cols(int K, int L, int P) {
 __host__ __device__ constexpr int tc_chunk(int L) { return L < 32 ? L : 32; }
 __host__ __device__ constexpr int tc_pitch(int L) { return tc_chunk(L) * 4 + 16; }
 __host__ __device__ constexpr size_t tc_stage_bytes(int L) { return (size_t)4 * 32 * tc_pitch(L); }
-__host__ __device__ constexpr size_t tc_td_bytes(int K, int L, int P) {
-  return (size_t)tc_nbuf(K, L, P) * kTcRows * P * tc_kt(K) * 4 + (size_t)L * tc_kt(K) * 4;
+__host__ __device__ constexpr size_t tc_td_bytes(int K, int L) {
+  return (size_t)tc_nbuf(K, L) * kTcRows * tc_kt(K) * 4 + (size_t)L * tc_kt(K) * 4;
 }
-__host__ __device__ constexpr int tc_nstage(int K, int L, int P) {
-  return tc_td_bytes(K, L, P) + 2 * tc_stage_bytes(L) + 1024 <= (size_t)220 * 1024 ? 2 : 1;
+__host__ __device__ constexpr int tc_nstage(int K, int L) {
+  return tc_td_bytes(K, L) + 2 * tc_stage_bytes(L) + 1024 <= (size_t)220 * 1024 ? 2 : 1;
 }
 
 // Shared memory: NBUF T tiles (kTcRows x KT) and D^T (L x KT), tf32 K-major
 // 128B-swizzled, then the epilogue stages, plus 1 KB of alignment slack.
-__host__ __device__ constexpr size_t tc_smem_bytes(int K, int L, int P) {
-  return tc_td_bytes(K, L, P) + tc_nstage(K, L, P) * tc_stage_bytes(L) + 1024;
+__host__ __device__ constexpr size_t tc_smem_bytes(int K, int L) {
+  return tc_td_bytes(K, L) + tc_nstage(K, L) * tc_stage_bytes(L) + 1024;
 }
 
 #ifndef SLNR_TC_BATCH
@@ -680,19 +672,6 @@ struct Placer {
   __device__ __forceinline__ void put(int slot, const float (&acc)[VPL]) {
     store_t_part<VPL>(tc_tiles() + ((slot / kTcRows) % NBUF) * TBYTES, slot % kTcRows, col, acc);
   }
-  // hi parts in columns [0, KT), lo parts in [KT, 2 KT)
-  template <int KT>
-  __device__ __forceinline__ void put_split(int slot, const float (&x)[VPL]) {
-    float hi[VPL], lo[VPL];
-#pragma unroll
-    for (int e = 0; e < VPL; ++e) {
-      hi[e] = __uint_as_float(tc::to_tf32(x[e]));
-      lo[e] = x[e] - hi[e];
-    }
-    uint8_t* t = tc_tiles() + ((slot / kTcRows) % NBUF) * TBYTES;
-    store_t_part<VPL>(t, slot % kTcRows, col, hi);
-    store_t_part<VPL>(t, slot % kTcRows, KT + col, lo);
-  }
   __device__ __forceinline__ void put_dest(int slot, int2 d) { g_tc.dest[(slot / kTcRows) % NBUF][slot % kTcRows] = d; }
   // The rows (and destinations) of slots [sl, sl + n), all in one slot tile,
   // are stored: make them visible to the tensor cores and count them on the
@@ -743,15 +722,14 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   static_assert(L % 16 == 0 && L >= 16 && L <= 256, "L must be a multiple of 16 in [16, 256]");
   constexpr int KT = tc_kt(K);  // tile columns (K, or 32 with zero padding)
   using PL = ProdLayout<K, MODE == kSampled>;
-  constexpr int P = tc_parts(MODE);
-  constexpr int NBUF = tc_nbuf(K, L, P);
+  constexpr int NBUF = tc_nbuf(K, L);
   constexpr uint32_t IDESC = tc::idesc_tf32(kTcRows, L);
   // TMEM columns: NBUF fp32 accumulators of L columns; an allocation is a
   // power of two of at least 32 columns
-  constexpr uint32_t NCOLS = tc_tmem_cols(K, L, P);
+  constexpr uint32_t NCOLS = tc_tmem_cols(K, L);
   static_assert(NCOLS >= (uint32_t)(NBUF * L) && NCOLS >= 32 && (NCOLS & (NCOLS - 1)) == 0 && NCOLS <= 512,
                 "tensor memory allocation");
-  constexpr int TBYTES = kTcRows * P * KT * 4;
+  constexpr int TBYTES = kTcRows * KT * 4;
   constexpr int CPT = kTcRows / PL::IPC;  // claims per item tile
   static_assert(NBUF <= kMaxBuf, "buffers");
   uint8_t* sT = tc_tiles();
@@ -782,7 +760,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   // with g_tc.tile_seq = j + 1 once written); the first local tile whose index
   // lies past the last item tile is g_tc.end_tile, and every role stops there.
   int nitems;  // < 2^31: segments or rows
-  if (!tc_dense_mode(MODE)) {
+  if (MODE != kDense) {
     const int n = hdr->n_segs;
     nitems = n < max_segs ? n : max_segs;
   } else {
@@ -810,9 +788,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   if constexpr (KT > K) {  // the padding columns of every T buffer: zero once, never written
     for (int i = tid; i < NBUF * kTcRows * (KT - K); i += kTcThreads) {
       const int b = i / (kTcRows * (KT - K)), r = (i / (KT - K)) % kTcRows, k = K + i % (KT - K);
-#pragma unroll
-      for (int h = 0; h < P; ++h)
-        *reinterpret_cast<uint32_t*>(sT + b * TBYTES + tc::sw128_offset(r, h * KT + k, kTcRows)) = 0u;
+      *reinterpret_cast<uint32_t*>(sT + b * TBYTES + tc::sw128_offset(r, k, kTcRows)) = 0u;
     }
   }
   tc::fence_proxy_async_smem();
@@ -869,16 +845,16 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       if (*reinterpret_cast<volatile int*>(&g_tc.fail_flag) != 0) break;  // another role timed out
       const int item0 = gid * kTcRows + (c % CPT) * PL::IPC + g * R;  // this group's first item
       bool ok = true;
-      if constexpr (tc_dense_mode(MODE)) {
-        // R rows of the materialised T (or of X), all loads in flight at once
+      if constexpr (MODE == kDense) {
+        // R rows of the materialised T, all loads in flight at once
         float x[R][VPL];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          if (item0 + r < nitems) gathered_row<K, VPL, MODE == kSplitH>(x[r], X, X2, item0 + r, col); else zero_vec(x[r]);
+          if (item0 + r < nitems) ldg_vec<VPL>(x[r], X + (int64_t)(item0 + r) * K + col); else zero_vec(x[r]);
         }
         const int sl = pl.take(R);
         ok = sl >= 0 && pl.template place<R>(sl, [&](int r, int slot) {
-          if constexpr (P == 2) pl.template put_split<KT>(slot, x[r]); else pl.put(slot, x[r]);
+          pl.put(slot, x[r]);
           if (gl == r) pl.put_dest(slot, make_int2(item0 + r < nitems ? item0 + r : -1, -1));
         });
       } else {
@@ -939,11 +915,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         tc::tc_fence_after_sync();
         const uint32_t a_base = sT_addr + b * TBYTES;
 #pragma unroll
-        for (int kb = 0; kb < P * KT / 32; ++kb)
+        for (int kb = 0; kb < KT / 32; ++kb)
 #pragma unroll
           for (int ks = 0; ks < 4; ++ks) {
             const uint64_t ad = tc::desc_k_sw128(a_base + kb * kTcRows * 128 + ks * 32);
-            const uint64_t bd = tc::desc_k_sw128(sD_addr + (kb % (KT / 32)) * L * 128 + ks * 32);
+            const uint64_t bd = tc::desc_k_sw128(sD_addr + kb * L * 128 + ks * 32);
             tc::mma_tf32(tmem + (uint32_t)(b * L), ad, bd, IDESC, (kb | ks) != 0);
           }
         tc::mma_commit(&g_tc.mma_bar[b]);
@@ -954,8 +930,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   } else {
     // ---------------- epilogue ----------------
     const int q = warp & 3;  // TMEM lane quadrant of this warp
-    constexpr int CW = tc_chunk(L), PITCH = tc_pitch(L), NSTAGE = tc_nstage(K, L, P);
-    uint8_t* stage = sT + tc_td_bytes(K, L, P) + (size_t)q * NSTAGE * 32 * PITCH;
+    constexpr int CW = tc_chunk(L), PITCH = tc_pitch(L), NSTAGE = tc_nstage(K, L);
+    uint8_t* stage = sT + tc_td_bytes(K, L) + (size_t)q * NSTAGE * 32 * PITCH;
     int stage_i = 0;
     for (int j = 0;; ++j) {
       const int b = j % NBUF;
@@ -1044,10 +1020,10 @@ cudaError_t tc_setup(TcLaunch* out) {
   int sm_smem = 0, nsm = 0;
   if ((e = cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  size_t smem = tc_smem_bytes(K, L, tc_parts(MODE));
+  size_t smem = tc_smem_bytes(K, L);
   // no more resident CTAs per SM than tensor memory (512 columns) holds
   // accumulators for: a CTA waiting in tcgen05.alloc would only idle
-  const int max_ctas = 512 / (int)tc_tmem_cols(K, L, tc_parts(MODE));
+  const int max_ctas = 512 / (int)tc_tmem_cols(K, L);
   const size_t floor_bytes = (size_t)sm_smem / (size_t)(max_ctas + 1) + 1;
   if (smem < floor_bytes) smem = floor_bytes;
   if ((e = cudaFuncSetAttribute(k_tc_gemm<K, L, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
@@ -1081,9 +1057,7 @@ cudaError_t tc_dispatch(int K, int L, int64_t items_upper, WsHeader* hdr, const 
     int64_t grid = (items_upper + kTcRows - 1) / kTcRows;                                                 \
     if (grid > tl.grid_cap) grid = tl.grid_cap;                                                           \
     if (grid < 1) grid = 1;                                                                               \
-    if (MODE != kSplit && MODE != kSplitH &&                                                             \
-        (e = cudaMemsetAsync(&hdr->next_tile, 0, sizeof(int), s)) != cudaSuccess)                         \
-      return e;                                                                                           \
+    if ((e = cudaMemsetAsync(&hdr->next_tile, 0, sizeof(int), s)) != cudaSuccess) return e;               \
     k_tc_gemm<KK, LL, MODE><<<SLNR_COUNTED((unsigned)grid), kTcThreads, tl.smem, s>>>(hdr, segs, max_segs, dense_rows,  \
                                                                          crd, vals, X, X2, Cq, D, A,     \
                                                                          partial, wait);                 \
@@ -1093,13 +1067,6 @@ cudaError_t tc_dispatch(int K, int L, int64_t items_upper, WsHeader* hdr, const 
     SLNR_TC_CASE(32, 32) SLNR_TC_CASE(32, 64) SLNR_TC_CASE(32, 128)
     SLNR_TC_CASE(64, 32) SLNR_TC_CASE(64, 64) SLNR_TC_CASE(64, 128)
     SLNR_TC_CASE(128, 32) SLNR_TC_CASE(128, 64) SLNR_TC_CASE(128, 128)
-    return cudaErrorInvalidValue;
-  }
-  if constexpr (tc_parts(MODE) == 2) {  // the widths whose two-part tile and D^T fit (tc_split_supported)
-    SLNR_TC_CASE(16, 16) SLNR_TC_CASE(16, 32) SLNR_TC_CASE(16, 64) SLNR_TC_CASE(16, 128)
-    SLNR_TC_CASE(32, 16) SLNR_TC_CASE(32, 32) SLNR_TC_CASE(32, 64) SLNR_TC_CASE(32, 128)
-    SLNR_TC_CASE(64, 16) SLNR_TC_CASE(64, 32) SLNR_TC_CASE(64, 64) SLNR_TC_CASE(64, 128)
-    SLNR_TC_CASE(128, 16) SLNR_TC_CASE(128, 32) SLNR_TC_CASE(128, 64) SLNR_TC_CASE(128, 128)
     return cudaErrorInvalidValue;
   }
   SLNR_TC_CASE(16, 16) SLNR_TC_CASE(16, 32) SLNR_TC_CASE(16, 64) SLNR_TC_CASE(16, 128) SLNR_TC_CASE(16, 256)
@@ -1116,13 +1083,8 @@ cudaError_t tc_dispatch(int K, int L, int64_t items_upper, WsHeader* hdr, const 
 bool tc_supported(int K, int L) {
   return (K == 16 || K == 32 || K == 64 || K == 128 || (K == 256 && L <= 64)) &&
          (L == 16 || L == 32 || L == 64 || L == 128 || L == 256) &&
-         tc_smem_bytes(K, L, 1) <= (size_t)220 * 1024;
+         tc_smem_bytes(K, L) <= (size_t)220 * 1024;
 }
-
-bool tc_split_supported(int K, int L) {
-  return (K == 16 || K == 32 || K == 64 || K == 128) && (L == 16 || L == 32 || L == 64 || L == 128);
-}
-static_assert(tc_smem_bytes(128, 128, 2) <= (size_t)220 * 1024, "the widest two-part tile fits");
 
 int seg_scan_blocks(int64_t nrows) { return (int)((nrows + kScanRows - 1) / kScanRows); }
 
@@ -1160,14 +1122,6 @@ cudaError_t launch_tc_sddmm_spmm_gemm(const CsrView& B, const float* C, const fl
   // T rows of width L: the gathered row is F(j,:), its scale C(i,:).D(j,:)
   return tc_dispatch<kSampled>(L, M, plan.max_segs, plan.hdr, plan.segs, plan.max_segs, 0, B.crd, B.vals, F, D, C,
                                W, A, plan.partial, s);
-}
-
-cudaError_t launch_tc_premul(int64_t M, int K, int L, const float* X, const float* X2, const float* D, float* G,
-                             WsHeader* hdr, cudaStream_t s) {
-  if (M <= 0) return cudaSuccess;
-  if (X2 != nullptr)
-    return tc_dispatch<kSplitH>(K, L, M, hdr, nullptr, 0, M, nullptr, nullptr, X, X2, nullptr, D, G, nullptr, s);
-  return tc_dispatch<kSplit>(K, L, M, hdr, nullptr, 0, M, nullptr, nullptr, X, nullptr, nullptr, D, G, nullptr, s);
 }
 
 cudaError_t launch_tc_dense_gemm(int64_t M, int K, int L, const float* T, const float* D, float* A,

@@ -138,6 +138,53 @@ def test_split_product_error(slnr, K, L, two):
     assert P.rel_err(out.cpu().numpy(), ref, ref_abs) <= 1e-5
 
 
+def columns_workload(ncols, K, L, two, positive=False):
+    """A graph over `ncols` columns with enough nonzeros for the tensor cores (2^14) and for each column."""
+    per = min(ncols, 30)
+    n = max(20000, ncols + 2000) // per + 1
+    r = wl.Rng(0x51A4 + ncols + K + L)
+    crd = np.concatenate([np.sort(np.random.default_rng(i).choice(ncols, per, replace=False)) for i in range(n)])
+    lo = 0.5 if positive else -1
+    B = wl.CSR(n, ncols, np.arange(n + 1, dtype=np.int32) * per, crd.astype(np.int32), wl.uniform(r, per * n, lo, 1))
+    X, X2 = wl.uniform(r, (ncols, K), lo, 1), wl.uniform(r, (ncols, K), lo, 1)
+    D = np.round(wl.uniform(r, (K, L), lo, 1) * 512).astype(np.float32) / 512
+    if two:
+        return wl.Workload("columns", "spmmh_gemm", B, {"C": X, "D": X2, "E": D}, {"J": K, "L": L})
+    return wl.Workload("columns", "spmm_gemm", B, {"C": X, "D": D}, {"K": K, "L": L})
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("two", [False, True])
+@pytest.mark.parametrize("ncols,K,L", [(1, 16, 16), (127, 128, 128), (128, 32, 64), (129, 128, 16), (8 * 30 + 1, 16, 32),
+                                       (130000, 128, 128), (40000, 64, 64), (19457, 32, 16)])
+def test_split_product_rows(slnr, ncols, K, L, two):
+    # one tile, its edges, one tile more than a CTA each, several tiles per CTA; the bound is the one above
+    w = columns_workload(ncols, K, L, two)
+    ref, ref_abs = oracle.get().run(w)
+    dB, dd = P.to_device(w)
+    out = slnr.run(w.op, dB, dd, allow_tf32=True)
+    assert P.rel_err(out.cpu().numpy(), ref, ref_abs) <= 1e-5
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("where", ["C", "D"])
+def test_split_product_infinities(slnr, where):
+    # positive values, some exact in tf32 (their second part is zero): an
+    # infinity stays one, and reaches the entries that it contributes to
+    w = columns_workload(500, 64, 64, False, positive=True)
+    w.dense["C"][::2] = 0.5
+    w.dense[where][3, 5] = np.inf
+    dB, dd = P.to_device(w)
+    out = slnr.run(w.op, dB, dd, allow_tf32=True).cpu().numpy()
+    if where == "D":
+        hit = np.zeros_like(out, dtype=bool)
+        hit[:, 5] = True
+    else:
+        rows = np.array([3 in w.B.crd[w.B.pos[i]:w.B.pos[i + 1]] for i in range(w.B.nrows)])
+        hit = np.repeat(rows[:, None], 64, axis=1)
+    assert np.array_equal(np.isposinf(out), hit) and np.isfinite(out[~hit]).all()
+
+
 def csf(kind, rng, d1, d2, seed):
     """CSF tensors whose slices and fibers end at window edges, span many windows, or are empty in runs."""
     if kind == "few":            # fewer nonzeros than a window
