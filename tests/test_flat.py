@@ -138,6 +138,30 @@ def test_split_product_error(slnr, K, L, two):
     assert P.rel_err(out.cpu().numpy(), ref, ref_abs) <= 1e-5
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("K,L", [(16, 16), (64, 32), (128, 128), (48, 12)])
+@pytest.mark.parametrize("runs", [[0], [1, 2], [3, 4, 5, 9], [63, 64, 65, 700], [5000, 0, 0, 70000]])
+def test_premultiplied_empty_rows(slnr, K, L, runs):
+    # runs of empty rows shorter and longer than the window kernel's steps, also after the last nonzero;
+    # fp32 sums of 3 products of K terms: below 1e-5 of the absolute sum
+    lens, ncols = [], 120
+    for i in range(0, 400 if max(runs) < 1000 else 12):
+        lens += [1 + i % 3] + [0] * runs[i % len(runs)]
+    lens += [40, 0, 0]
+    pos = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    r = wl.Rng(0x51A4 + K + L + len(lens))
+    crd = np.concatenate([np.sort(np.random.default_rng(i).choice(ncols, n, replace=False))
+                          for i, n in enumerate(lens) if n]).astype(np.int32)
+    B = wl.CSR(len(lens), ncols, pos, crd, wl.uniform(r, int(pos[-1]), -1, 1))
+    w = wl.Workload("empty", "spmm_gemm", B, {"C": wl.uniform(r, (ncols, K), -1, 1), "D": wl.uniform(r, (K, L), -1, 1)},
+                    {"K": K, "L": L})
+    ref, ref_abs = oracle.get().run(w)
+    dB, dd = P.to_device(w)
+    out = slnr.run(w.op, dB, dd, allow_tf32=False).cpu().numpy()
+    assert P.rel_err(out, ref, ref_abs) <= 1e-5
+    assert not out[np.diff(pos) == 0].any()
+
+
 def columns_workload(ncols, K, L, two, positive=False):
     """A graph over `ncols` columns with enough nonzeros for the tensor cores (2^14) and for each column."""
     per = min(ncols, 30)
