@@ -323,11 +323,16 @@ bool use_tc_fused(const slnr_opts* o, int32_t K, int32_t L, int64_t nnz) {
 //    large call (2.5M 32/128 119 | 134);
 //  - sampled rows: row first where D widens them (R-MAT 718k rows 16/16/64
 //    825 | 1142, uniform 39k 16/16/128 40 | 48);
-//  - tensor cores: D first on graphs of fewer rows, where the row kernel's
-//    tiles of heavy rows set its time (50k rows 128/128 159 | 90, 220k 64/64
-//    201 | 128), row first on larger ones (500k 32/32 118 | 160, 1M 128/128
-//    940 | 1000) and where D widens the rows (220k 32/128 107 | 154); two
-//    gathered matrices move the line up (1M 128/128 1750 | 1077).
+//  - tensor cores: uniform graphs gain from D first nearly throughout, R-MAT
+//    graphs lose where the rows are narrow or many (heavy rows and long runs of
+//    empty ones), and the sizes do not tell them apart: D first where neither
+//    is slower.  Up to 40k rows at K = 16 (30k: uniform 41 | 31, R-MAT 69 | 64;
+//    100k: 56 | 37, 70 | 110), 64k at K = 32 (50k R-MAT 83 | 60, 400k 108 |
+//    150), 256k at K >= 64 (220k 64/64 R-MAT 200 | 118, uniform 85 | 62), 128k
+//    if D widens the rows (64/128 uniform 100k 92 | 84, 220k 166 | 220).  Of
+//    more rows, degrees of 14 (1M 128/128 914 | 840, uniform 1525 | 1379), or 8
+//    where D narrows them (500k 128/32 342 | 294).  Two gathered matrices move
+//    the line up (1M 128/128 1660 | 930).
 bool use_tc_premul(const slnr_opts* o, int32_t K, int32_t L, int64_t nnz) {
   return o->allow_tf32 != 0 && tc_split_supported(K, L) && nnz >= kTcFusedMinNnz;
 }
@@ -336,13 +341,14 @@ bool premul_first(const slnr_opts* o, PremulKind kind, int64_t nrows, int64_t nc
                   bool row_tc) {
   if (o->variant != SLNR_FUSED || nnz < 1 || nnz < ncols) return false;
   if (L > K && nnz > 64 * nrows) return false;  // long rows: the narrower rows are gathered
-  const int64_t k = 1024, few = (K <= 32 ? 128 : 256) * k;
+  const int64_t k = 1024;
   if (kind == kFibers) return !row_tc || L <= 2 * K || nnz < 2048 * k;
   if (kind == kSampledRows && L > 2 * K && nrows >= (L > 4 * K ? 0 : 64 * k)) return false;
   if (!row_tc) return L <= 4 * K || nnz < 256 * k;
-  if (L > 2 * K) return nrows < 64 * k;
-  if (kind == kTwo) return nrows < few || nnz >= 8 * nrows;
-  if (nrows >= few) return kind == kOne && K == 64 && L < 64 && nnz >= 8 * nrows;
+  if (L > 2 * K) return nrows < (K <= 16 && kind == kOne ? 40 * k : 64 * k);
+  if (kind == kTwo) return nrows < (K <= 32 ? 128 : 256) * k || nnz >= 8 * nrows;
+  const int64_t few = (K <= 32 && kind == kOne ? (K <= 16 ? 40 : 64) : K <= 32 || L > K ? 128 : 256) * k;
+  if (nrows >= few) return K >= 64 && L <= K && nnz >= (L < K ? 8 : 14) * nrows;
   return K < 128 || nrows < 64 * k || nnz >= 8 * nrows;
 }
 
