@@ -502,7 +502,7 @@ slnr_status premul_sum(const CsrView& v, const float* X, const float* X2, int32_
   if (tc) fp.hdr = nullptr;  // zeroed before the tensor-core kernel, which may raise a flag
   SLNR_CHECK(premul(v.ncols, K, L, X, X2, D, G, ws, tc, s));
   SLNR_LAUNCH("flat_rows", launch_flat_rows(v, L, A, fp, s));
-  SLNR_LAUNCH("flat_sum", launch_flat_sum(v, G, nullptr, L, A, fp, s));
+  SLNR_LAUNCH("flat_sum", launch_flat_sum(v, G, L, A, fp, s));
   return SLNR_OK;
 }
 

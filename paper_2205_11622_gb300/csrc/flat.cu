@@ -2,7 +2,6 @@
 // output row is a weighted sum of gathered rows:
 //
 //   kSum       out(r,:) = sum_p vals[p] X(crd[p],:)
-//   kSumH      out(r,:) = sum_p vals[p] X(crd[p],:) .* X2(crd[p],:)
 //   kSampled   out(r,:) = sum_p vals[p] <C(r,:), D(crd[p],:)> X(crd[p],:)
 //              (fused <SDDMM,SpMM>, Fig. 2d: the scalar of each stored (i,j)
 //              is formed and used at once)
@@ -31,7 +30,7 @@ namespace {
 using flat::Row;
 using flat::u64;
 
-enum FlatMode { kSum = 0, kSumH = 1, kSampled = 2 };
+enum FlatMode { kSum = 0, kSampled = 1 };
 
 constexpr int kFlatThreads = 128;
 constexpr int kFlatSms = 152;  // the window sizes are for this many SMs (sizes only: no device is asked)
@@ -99,7 +98,7 @@ struct FlatArgs {
   const int32_t* crd;
   const float* vals;
   const float* X;
-  const float* X2;  // kSumH: the second factor; kSampled: D
+  const float* D;   // kSampled
   const float* C;   // kSampled
   int W;            // width of X and out
   int L;            // kSampled: width of C and D
@@ -166,7 +165,7 @@ struct FlatPtrs {
   using Ptr = flat::RowPtr<GS, NCH, KIND>;
   Ptr x, d, c, out;
   __device__ __forceinline__ FlatPtrs(const FlatArgs& a, int gl)
-      : x(a.X, a.W, gl), d(a.X2, MODE == kSampled ? a.L : a.W, gl), c(a.C, a.L, gl), out(a.out, a.W, gl) {}
+      : x(a.X, a.W, gl), d(a.D, a.L, gl), c(a.C, a.L, gl), out(a.out, a.W, gl) {}
 };
 
 // U nonzeros of each window of the warp, entries e0 .. e0 + U - 1 of this
@@ -218,7 +217,6 @@ __device__ __forceinline__ void flat_batch(const FlatPtrs<GS, NCH, MODE, KIND>& 
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      if constexpr (MODE == kSumH) x[u].mul(d[u]);
       acc.fma(flat::pack2(val[u]), x[u]);
     }
     return;
@@ -271,7 +269,6 @@ __device__ __forceinline__ void flat_batch(const FlatPtrs<GS, NCH, MODE, KIND>& 
     }
     float v = val[u];
     if constexpr (MODE == kSampled) v *= group_sum<GS>(R::dot_part(m.d, c, d[u]));
-    if constexpr (MODE == kSumH) x[u].mul(d[u]);
     if (u < live) acc.fma(flat::pack2(v), x[u]);
   }
 }
@@ -517,7 +514,7 @@ cudaError_t flat_run(const FlatArgs& a, cudaStream_t s) {
   if (a.nrows <= 0) return cudaSuccess;
   const int wm = MODE == kSampled && a.L > a.W ? a.L : a.W;
   // 32-byte accesses where every row of every operand allows them
-  const bool v8 = a.W % 8 == 0 && aligned32(a.X) && aligned32(a.out) && aligned32(a.X2) && aligned32(a.C) &&
+  const bool v8 = a.W % 8 == 0 && aligned32(a.X) && aligned32(a.out) && aligned32(a.D) && aligned32(a.C) &&
                   (MODE != kSampled || a.L % 8 == 0);
   if (!v8) return flat_width<MODE, flat::kV4>(wm, a, s);
   const bool whole = wm >= 8 && (wm & (wm - 1)) == 0 && (MODE != kSampled || a.L == a.W);
@@ -555,19 +552,17 @@ cudaError_t launch_flat_rows(const CsrView& B, int W, float* out, const FlatPlan
   return cudaGetLastError();
 }
 
-cudaError_t launch_flat_sum(const CsrView& B, const float* X, const float* X2, int W, float* out, const FlatPlan& plan,
-                            cudaStream_t s) {
+cudaError_t launch_flat_sum(const CsrView& B, const float* X, int W, float* out, const FlatPlan& plan, cudaStream_t s) {
   FlatArgs a = flat_args(B, W, out, plan);
   a.X = X;
-  a.X2 = X2;
-  return X2 == nullptr ? flat_run<kSum>(a, s) : flat_run<kSumH>(a, s);
+  return flat_run<kSum>(a, s);
 }
 
 cudaError_t launch_flat_sampled(const CsrView& B, const float* C, const float* D, int L, const float* E, int K,
                                 float* out, const FlatPlan& plan, cudaStream_t s) {
   FlatArgs a = flat_args(B, K, out, plan);
   a.X = E;
-  a.X2 = D;
+  a.D = D;
   a.C = C;
   a.L = L;
   return flat_run<kSampled>(a, s);

@@ -178,10 +178,6 @@ struct Row {
 #pragma unroll
     for (int i = 0; i < P; ++i) v[i] = fma2(s, x.v[i], v[i]);
   }
-  __device__ __forceinline__ void mul(const Row& x) {
-#pragma unroll
-    for (int i = 0; i < P; ++i) v[i] = mul2(v[i], x.v[i]);
-  }
   __device__ __forceinline__ void add(const Row& x) {
 #pragma unroll
     for (int i = 0; i < P; ++i) v[i] = add2(v[i], x.v[i]);

@@ -148,9 +148,8 @@ cudaError_t launch_tc_sddmm_spmm_gemm(const CsrView& B, const float* C, const fl
 // (sampled: for launch_flat_sampled).
 int flat_window(int64_t nnz, int wm, bool sampled);
 cudaError_t launch_flat_rows(const CsrView& B, int W, float* out, const FlatPlan& plan, cudaStream_t s);
-// out = B . X (with X2 not NULL the gathered row is X .* X2)
-cudaError_t launch_flat_sum(const CsrView& B, const float* X, const float* X2, int W, float* out, const FlatPlan& plan,
-                            cudaStream_t s);
+// out = B . X
+cudaError_t launch_flat_sum(const CsrView& B, const float* X, int W, float* out, const FlatPlan& plan, cudaStream_t s);
 // fused <SDDMM,SpMM>: C nrows x L, D ncols x L, E ncols x K
 cudaError_t launch_flat_sampled(const CsrView& B, const float* C, const float* D, int L, const float* E, int K,
                                 float* out, const FlatPlan& plan, cudaStream_t s);
