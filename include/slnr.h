@@ -9,7 +9,12 @@
  * (Sec. 4.2, Algorithm 1) derives: the outer sparse loop (CSR row, or CSF
  * slice / fiber) is shared by the producer and the consumer, the producer
  * fills a small temporary (a scalar or a vector) and the consumer uses it at
- * once, so the intermediate tensor is never written to memory.  Each entry
+ * once, so the intermediate tensor is never written to memory.  Where a vector
+ * temporary is multiplied by a dense matrix, the library may take the product
+ * in the other order, by sizes and widths alone: the dense matrices first, once
+ * per gathered row into the workspace, then the sparse sum (the same sums in
+ * another order; with infinite or overflowing values the two orders can differ
+ * in what is infinite and what is NaN).  Each entry
  * point also has an UNFUSED variant that materialises the intermediate in the
  * caller's workspace and runs producer and consumer as separate kernels (the
  * paper's "TACO Separate" baseline, Sec. 6); slnr_spmm_gemm_original runs
@@ -134,9 +139,10 @@ slnr_status slnr_spmmh_gemm_workspace(const slnr_csr *B, int32_t J, int32_t L, c
  * A(i,l) = sum_{j,k} B(i,j) * C(j,k) * D(k,l)
  *   B: nrows x ncols CSR.  C: ncols x K.  D: K x L.  A: nrows x L (output).
  * Fused: per row i, the temporary T(k) = sum_j B(i,j) C(j,k) is built on chip
- * and multiplied by D at once (the vector temporary over k of Sec. 6.3).
+ * and multiplied by D at once (the vector temporary over k of Sec. 6.3); or
+ * C.D (ncols x L) is formed in the workspace and its rows are summed into A.
  * Unfused: T = B.C is written to the workspace (nrows x K), then A = T.D.
- * With allow_tf32 the T.D contraction may use TF32 tensor cores. */
+ * With allow_tf32 the contraction with D may use TF32 tensor cores. */
 slnr_status slnr_spmm_gemm(const slnr_csr *B, const float *C, int32_t K, const float *D, int32_t L,
                            float *A, const slnr_opts *opts);
 
@@ -167,9 +173,10 @@ slnr_status slnr_mttkrp(const slnr_csf3 *B, const float *C, const float *D, int3
  *   (A_pos1[2], A_crd1[nslices], A_pos2[nslices+1], A_crd2[nfibers]), and
  *   A_vals (nfibers x M, row f belongs to B's fiber f).
  * Fused: per fiber the temporary T(l) = sum_k B(i,j,k) C(k,l) is built on chip
- * and multiplied by D at once.  Unfused ("separate1" of Sec. 6.2): T for every
+ * and multiplied by D at once; or C.D (d2 x M) is formed in the workspace and
+ * its rows are summed.  Unfused ("separate1" of Sec. 6.2): T for every
  * fiber is written to the workspace, then A_vals = T.D.  With allow_tf32 the
- * T.D contraction may use TF32 tensor cores. */
+ * contraction with D may use TF32 tensor cores. */
 slnr_status slnr_spttm_ttm(const slnr_csf3 *B, const float *C, int32_t L, const float *D, int32_t M,
                            int32_t *A_pos1, int32_t *A_crd1, int32_t *A_pos2, int32_t *A_crd2,
                            float *A_vals, const slnr_opts *opts);
@@ -182,7 +189,9 @@ slnr_status slnr_spttm_ttm(const slnr_csf3 *B, const float *C, int32_t L, const 
  * y = B(i,j) C(i,:).D(j,:) is formed and T(i,:) += y F(j,:) at once; the row's
  * vector temporary T(i,:) (length L) stays on chip and A(i,:) = T(i,:).W
  * follows: on TF32 tensor cores with allow_tf32 when K == L in {32, 64, 128}
- * and M in {32, 64, 128}, else fp32 FFMA.  Unfused: the sampled product Y (nnz values) and
+ * and M in {32, 64, 128}, else fp32 FFMA; or F.W (ncols x M) is formed in the
+ * workspace (on TF32 tensor cores with allow_tf32 where the widths allow) and
+ * each y adds a row of it to A.  Unfused: the sampled product Y (nnz values) and
  * T = Y.F (nrows x L) are written to the workspace, then A = T.W (TF32 tensor
  * cores with allow_tf32, where the widths allow). */
 slnr_status slnr_sddmm_spmm_gemm(const slnr_csr *B, const float *C, const float *D, int32_t K, const float *F,
@@ -193,8 +202,8 @@ slnr_status slnr_sddmm_spmm_gemm(const slnr_csr *B, const float *C, const float 
  *   B: d0 x d1 x d2 CSF.  C: d1 x L.  D: d2 x L.  E: L x M.  A: d0 x M (output).
  *   (The paper writes the rank index as j: A_im = sum B_ikl C_lj D_kj E_jm.)
  * Fused: as slnr_mttkrp, and each slice's MTTKRP row u(i,:) (length L) is
- * formed on chip and multiplied by E at once (fp32 FFMA); rows without a
- * slice are zero.  Unfused: the MTTKRP result (d0 x L) is written to the
+ * written to the workspace (nslices x L) and multiplied by E (fp32 FFMA);
+ * rows without a slice are zero.  Unfused: the MTTKRP result (d0 x L) is written to the
  * workspace (itself by the unfused MTTKRP schedule), then A = result.E. */
 slnr_status slnr_mttkrp_gemm(const slnr_csf3 *B, const float *C, const float *D, int32_t L, const float *E,
                              int32_t M, float *A, const slnr_opts *opts);
@@ -204,7 +213,8 @@ slnr_status slnr_mttkrp_gemm(const slnr_csf3 *B, const float *C, const float *D,
  *   B: nrows x ncols CSR.  C, D: ncols x J.  E: J x L.  A: nrows x L (output).
  * Fused: per row i the temporary T(j) = sum_k B(i,k) C(k,j) D(k,j) (a sparse
  * row times the Hadamard product of the gathered rows) is built on chip and
- * multiplied by E at once, as in <SpMM,GEMM>.  Unfused: T (nrows x J) is
+ * multiplied by E at once; or (C .* D).E (ncols x L) is formed in the
+ * workspace and its rows are summed, as in <SpMM,GEMM>.  Unfused: T (nrows x J) is
  * written to the workspace, then A = T.E.  With allow_tf32 the T.E
  * contraction may use TF32 tensor cores. */
 slnr_status slnr_spmmh_gemm(const slnr_csr *B, const float *C, const float *D, int32_t J, const float *E,
