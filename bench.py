@@ -177,19 +177,30 @@ def consumer_flops(w) -> int:
     return 0
 
 
-def gather_bytes(w) -> int:
-    """Bytes the fused producers read as whole gathered rows, one (or two)
+def gather_bytes(w, product_first=False) -> int:
+    """Bytes the fused kernels read as whole gathered rows, one (or two)
     per nonzero and one per fiber where a fiber scales a row: nnz 4K for
     <SpMM,GEMM>, nnz 4L for <SpTTM,SpTTM>, nnz 8J for <SpMMH,GEMM>, nnz 4(L+K)
     for <SDDMM,SpMM>, nnz 4(K+L) for <SDDMM,SpMM,GEMM>, (nnz + nfibers) 4L for
-    MTTKRP.  Almost all of them hit in L2; their rate, not HBM's, is the
+    MTTKRP.  Where the dense product comes first (product_first), a row of that
+    product takes the place of the gathered operands: nnz 4L, or 4M for
+    <SpTTM,SpTTM>.  Almost all of them hit in L2; their rate, not HBM's, is the
     realistic ceiling of the gathering kernels."""
     d, B = w.dims, w.B
+    if product_first:
+        return int(4 * d["M" if w.op == "spttm_ttm" else "L"] * B.nnz)
     per_nnz = {"spmm_gemm": lambda: 4 * d["K"], "spttm_ttm": lambda: 4 * d["L"], "spmmh_gemm": lambda: 8 * d["J"],
                "sddmm_spmm": lambda: 4 * (d["L"] + d["K"]), "sddmm_spmm_gemm": lambda: 4 * (d["K"] + d["L"]),
                "mttkrp": lambda: 4 * d["L"], "mttkrp_gemm": lambda: 4 * d["L"]}[w.op]()
     extra = 4 * d["L"] * B.nfibers if w.op in ("mttkrp", "mttkrp_gemm") else 0
     return int(per_nnz * B.nnz + extra)
+
+
+def dense_product_shape(w):
+    """(K, L) of the expression's contraction with a dense matrix."""
+    d = w.dims
+    return {"spmm_gemm": lambda: (d["K"], d["L"]), "spmmh_gemm": lambda: (d["J"], d["L"]),
+            "spttm_ttm": lambda: (d["L"], d["M"]), "sddmm_spmm_gemm": lambda: (d["L"], d["M"])}[w.op]()
 
 
 def gather_row_width(w) -> int:
@@ -558,8 +569,13 @@ def main():
     all_rows = min_bytes_all_rows(dw)
     traffic = ncu_traffic(dw.name)
     pk = slnr.peaks(stream, gather_width=gather_row_width(dw)) if rank == 0 else {}
-    gb = gather_bytes(dw)
-    cflops = consumer_flops(dw)
+    gb = gather_bytes(dw, product_first=kname == "flat_sum")
+    cflops, c_ms = consumer_flops(dw), k_ms
+    for name in ("tc_premul", "premul"):  # the dense product first: once per column, in a launch of its own
+        if name in kern_ms[dom]:
+            K, L = dense_product_shape(dw)
+            cols = dw.B.dims[2] if dw.op == "spttm_ttm" else dw.B.ncols
+            cflops, c_ms = 2 * cols * K * L, kern_ms[dom][name] / args.steps
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                 "frac": round(achieved / peak, 4), "traffic": traffic,
                 "kernel": f"{kname} of {dw.name} ({k_ms:.4f} ms per launch); achieved = the call's "
@@ -570,19 +586,21 @@ def main():
                 "frac_all_rows": round(all_rows / (k_ms / 1e3) / 1e9 / peak, 4),
                 "compute": {"unit": "TFLOP/s", "tf32_peak_measured": round(pk.get("tf32_tflops", 0.0), 1),
                             "ffma_peak_measured": round(pk.get("ffma_tflops", 0.0), 1),
-                            "tf32_achieved": round(cflops / (k_ms / 1e3) / 1e12, 2),
-                            "tf32_frac": round(cflops / (k_ms / 1e3) / 1e12 / pk["tf32_tflops"], 4)
+                            "tf32_achieved": round(cflops / (c_ms / 1e3) / 1e12, 2),
+                            "tf32_frac": round(cflops / (c_ms / 1e3) / 1e12 / pk["tf32_tflops"], 4)
                             if pk.get("tf32_tflops") else None,
-                            "note": "the dense consumer contraction of the dominant kernel (2 K L per non-empty "
-                                    "row) against this library's own tcgen05 kind::tf32 peak kernel"},
+                            "note": "the dense contraction (2 K L per non-empty row inside the dominant kernel, or "
+                                    "per column in its own launch) against this library's own tcgen05 kind::tf32 "
+                                    "peak kernel"},
                 "gather": {"bytes": gb, "unit": "GB/s", "achieved": round(gb / (k_ms / 1e3) / 1e9, 1),
                            "l2_gather_peak_measured": round(pk.get("l2_gather_gbs", 0.0), 1),
                            "hbm_gather_peak_measured": round(pk.get("hbm_gather_gbs", 0.0), 1),
                            "frac_l2": round(gb / (k_ms / 1e3) / 1e9 / pk["l2_gather_gbs"], 4)
                            if pk.get("l2_gather_gbs") else None,
                            "row_width": gather_row_width(dw),
-                           "note": "whole rows the producers gather (one per nonzero), against this library's own "
-                                   "row-gather kernel on an L2-resident table (a quarter of L2) and on a 2 GB table"}}
+                           "note": "whole rows the dominant kernel gathers (one or two per nonzero), against "
+                                   "this library's own row-gather kernel on an L2-resident table (a quarter "
+                                   "of L2) and on a 2 GB table"}}
 
     cpu = None
     if rank == 0 and world == 1 and not args.skip_cpu:
