@@ -327,28 +327,44 @@ bool use_tc_fused(const slnr_opts* o, int32_t K, int32_t L, int64_t nnz) {
 //    graphs lose where the rows are narrow or many (heavy rows and long runs of
 //    empty ones), and the sizes do not tell them apart: D first where neither
 //    is slower.  Up to 40k rows at K = 16 (30k: uniform 41 | 31, R-MAT 69 | 64;
-//    100k: 56 | 37, 70 | 110), 64k at K = 32 (50k R-MAT 83 | 60, 400k 108 |
-//    150), 256k at K >= 64 (220k 64/64 R-MAT 200 | 118, uniform 85 | 62), 128k
-//    if D widens the rows (64/128 uniform 100k 92 | 84, 220k 166 | 220).  Of
-//    more rows, degrees of 14 (1M 128/128 914 | 840, uniform 1525 | 1379), or 8
-//    where D narrows them (500k 128/32 342 | 294).  Two gathered matrices move
-//    the line up (1M 128/128 1660 | 930).
+//    100k: 56 | 37, 70 | 110), 64k at K = 32 (50k R-MAT 83 | 60), 128k at
+//    K >= 64, from 64k on at K >= 128 of degrees of 8 or more.  Two gathered
+//    matrices or sampled rows move the line up to 128k throughout.
 bool use_tc_premul(const slnr_opts* o, int32_t K, int32_t L, int64_t nnz) {
   return o->allow_tf32 != 0 && tc_split_supported(K, L) && nnz >= kTcFusedMinNnz;
 }
 enum PremulKind { kOne, kTwo, kSampledRows, kFibers };
+
+// Whether the two orders give nearly the same values where the row kernel runs
+// on the tensor cores.  It rounds T to tf32 once per segment of a row, D first
+// does not, so a row's values differ by 2.1e-4 of that row's size (2.9e-4 where
+// the product runs in fp32 and D is not rounded either).  Against the values of
+// the whole result that grows with the longest row's share: up to 5 such
+// deviations times the root of (longest row / mean row).  D first is left to
+// calls where that stays below 2e-2: fibers that cannot be 350 (175) times as
+// long as the mean one, and graphs of fewer than 128k (64k) rows.  Largest
+// difference of any value over the result's rms (or over itself where that is
+// larger), R-MAT graphs, 24 to 300 inputs each: under 128k rows 0.0137 (fp32,
+// under 64k rows, 0.0124); 250k 0.0207, 520k 0.0215, 1M 0.028; 5000-long modes
+// of fibers of mean 8 0.0246, modes of up to 2800 0.0110.
+bool premul_near(PremulKind kind, int64_t nrows, int64_t ncols, int64_t nnz, int32_t K, int32_t L) {
+  const bool rounded = tc_split_supported(K, L);
+  if (kind == kFibers) return ncols * nrows <= (rounded ? 350 : 175) * nnz;
+  return nrows < (rounded ? 128 : 64) * 1024;
+}
+
 bool premul_first(const slnr_opts* o, PremulKind kind, int64_t nrows, int64_t ncols, int64_t nnz, int32_t K, int32_t L,
                   bool row_tc) {
   if (o->variant != SLNR_FUSED || nnz < 1 || nnz < ncols) return false;
   if (L > K && nnz > 64 * nrows) return false;  // long rows: the narrower rows are gathered
+  if (row_tc && !premul_near(kind, nrows, ncols, nnz, K, L)) return false;
   const int64_t k = 1024;
   if (kind == kFibers) return !row_tc || L <= 2 * K || nnz < 2048 * k;
   if (kind == kSampledRows && L > 2 * K && nrows >= (L > 4 * K ? 0 : 64 * k)) return false;
   if (!row_tc) return L <= 4 * K || nnz < 256 * k;
   if (L > 2 * K) return nrows < (K <= 16 && kind == kOne ? 40 * k : 64 * k);
-  if (kind == kTwo) return nrows < (K <= 32 ? 128 : 256) * k || nnz >= 8 * nrows;
-  const int64_t few = (K <= 32 && kind == kOne ? (K <= 16 ? 40 : 64) : K <= 32 || L > K ? 128 : 256) * k;
-  if (nrows >= few) return K >= 64 && L <= K && nnz >= (L < K ? 8 : 14) * nrows;
+  if (kind == kTwo) return true;
+  if (kind == kOne && K <= 32 && nrows >= (K <= 16 ? 40 : 64) * k) return false;
   return K < 128 || nrows < 64 * k || nnz >= 8 * nrows;
 }
 

@@ -1,0 +1,140 @@
+"""Which contraction of A = B.X.D comes first, and that neither order costs a
+caller anything: values, precision, time-saving routes and workspace.
+
+D first (X.D once per row of X, then sums of its rows) and row first (T = B.X
+row by row on chip, times D) give the same sums in another order.  With TF32
+the row kernel rounds T once per segment of at most 128 nonzeros, which D first
+does not, so the calls that ran row first keep that order wherever a value could
+differ by more than 2e-2 of the result's root mean square.
+"""
+import ctypes
+
+import numpy as np
+import pytest
+
+import _parity as P
+import oracle
+import workloads as wl
+
+import paper_2205_11622_gb300 as slnr
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    slnr.build()
+    slnr.lib()
+
+
+def phases(w, B, dense, **kw):
+    """(output values, names of the call's phases)."""
+    slnr.timing_enable(True)
+    try:
+        out = slnr.run(w.op, B, dense, **kw)
+        names = [n for n, _ in slnr.timing_read()]
+    finally:
+        slnr.timing_enable(False)
+    assert slnr.device_flags() == 0
+    return P.values_of(w.op, out), names
+
+
+def csr_of(lens, ncols, seed):
+    """Rows of the given lengths: distinct columns a + b t mod ncols, sorted."""
+    rng = np.random.default_rng(seed)
+    coprime = [b for b in range(1, 200) if np.gcd(b, ncols) == 1]
+    crd = [np.sort((int(rng.integers(ncols)) + coprime[int(rng.integers(len(coprime)))] *
+                    np.arange(n, dtype=np.int64)) % ncols) for n in lens if n]
+    pos = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    crd = np.concatenate(crd or [[]]).astype(np.int32)
+    return wl.CSR(len(lens), ncols, pos, crd, wl.uniform(wl.Rng(seed), len(crd), -1, 1))
+
+
+def csf_of(lens, d2, seed, d1=40):
+    """Fibers of the given lengths, d1 of them to a slice."""
+    f = csr_of(lens, d2, seed)
+    nf = len(lens)
+    ns = -(-nf // d1)
+    pos2 = np.minimum(np.arange(ns + 1) * d1, nf).astype(np.int32)
+    return wl.CSF3((ns, d1, d2), np.array([0, ns], np.int32), np.arange(ns, dtype=np.int32), pos2,
+                   (np.arange(nf) % d1).astype(np.int32), f.pos, f.crd, f.vals)
+
+
+def workload(op, lens, ncols, K, L, seed):
+    """The call on rows (or fibers) of the given lengths: gathered width K, output width L."""
+    r = wl.Rng(seed + 1)
+    n = len(lens)
+    if op == "spttm_ttm":
+        return wl.Workload("order", op, csf_of(lens, ncols, seed),
+                           {"C": wl.normal(r, (ncols, K)), "D": wl.normal(r, (K, L))}, {"L": K, "M": L})
+    B = csr_of(lens, ncols, seed)
+    if op == "spmm_gemm":
+        return wl.Workload("order", op, B, {"C": wl.normal(r, (ncols, K)), "D": wl.normal(r, (K, L))}, {"K": K, "L": L})
+    if op == "spmmh_gemm":
+        return wl.Workload("order", op, B, {"C": wl.normal(r, (ncols, K)), "D": wl.normal(r, (ncols, K)),
+                                            "E": wl.normal(r, (K, L))}, {"J": K, "L": L})
+    return wl.Workload("order", op, B, {"C": wl.normal(r, (n, K)), "D": wl.normal(r, (ncols, K)),
+                                        "F": wl.normal(r, (ncols, K)), "W": wl.normal(r, (K, L))},
+                       {"K": K, "L": K, "M": L})
+
+
+def tf32(x):
+    """x rounded to 10 mantissa bits, halves away from zero."""
+    u = np.ascontiguousarray(x, np.float32).view(np.uint32)
+    return ((u + np.uint32(0x1000)) & np.uint32(0xFFFFE000)).view(np.float32).astype(np.float64)
+
+
+def row_first(w):
+    """The result with T rounded to tf32 once per segment of 128 nonzeros and D once, sums in fp64."""
+    d = w.dense
+    pos, crd = (w.B.pos3, w.B.crd3) if w.op == "spttm_ttm" else (w.B.pos, w.B.crd)
+    X = d["F"] if w.op == "sddmm_spmm_gemm" else d["C"]
+    consumer = {"spmm_gemm": "D", "spttm_ttm": "D", "spmmh_gemm": "E", "sddmm_spmm_gemm": "W"}[w.op]
+    v = w.B.vals.astype(np.float64)
+    rows = np.repeat(np.arange(len(pos) - 1), np.diff(pos))
+    if w.op == "sddmm_spmm_gemm":
+        v = v * np.einsum("pk,pk->p", d["C"][rows].astype(np.float64), d["D"][crd].astype(np.float64))
+    g = X[crd].astype(np.float64)
+    if w.op == "spmmh_gemm":
+        g *= d["D"][crd]
+    starts = np.concatenate([np.arange(a, b, 128) for a, b in zip(pos[:-1], pos[1:]) if a < b])
+    seg = np.add.reduceat(v[:, None] * g, starts, axis=0)
+    out = np.zeros((len(pos) - 1, d[consumer].shape[1]))
+    np.add.at(out, rows[starts], tf32(seg) @ tf32(d[consumer]))
+    return out
+
+
+# A row (fiber) of 50000 nonzeros among short ones: 200 times the root mean square length, so that D first
+# differs by 0.1 and more; the row kernel's own order of fp32 sums moves single roundings, 1e-3 at most.
+@pytest.mark.gpu
+@pytest.mark.parametrize("op,K,L", [("spmm_gemm", 64, 64), ("spmm_gemm", 128, 128), ("spmmh_gemm", 64, 32),
+                                    ("sddmm_spmm_gemm", 64, 64), ("spttm_ttm", 64, 64)])
+def test_tf32_values_stay_where_rows_are_long(gpu, op, K, L):
+    n, ncols = (3000, 50000) if op == "spttm_ttm" else (132000, 132000)
+    lens = np.full(n, 1)
+    lens[5] = 50000
+    w = workload(op, lens.tolist(), ncols, K, L, 0x51A4 + K)
+    B, dense = P.to_device(w)
+    got, _ = phases(w, B, dense, allow_tf32=True)
+    ref = row_first(w)
+    rms = np.sqrt(np.mean(ref ** 2))
+    assert np.max(np.abs(got.cpu().numpy() - ref) / np.maximum(rms, np.abs(ref))) <= 5e-3
+
+
+def csr_bytes(op, nrows, ncols, nnz, sizes, tf32=1):
+    n = ctypes.c_size_t(0)
+    B = slnr.slnr_csr(nrows, ncols, nnz, 0x1000, 0x2000, 0x3000)
+    o = slnr.slnr_opts(0, tf32, 0, 0, None, None, 0)
+    assert getattr(slnr.lib(), f"slnr_{op}_workspace")(ctypes.byref(B), *sizes, ctypes.byref(o), ctypes.byref(n)) == 0
+    return n.value
+
+
+@pytest.mark.parametrize("op,sizes", [("spmm_gemm", (64, 64)), ("spmm_gemm", (128, 128)), ("spmm_gemm", (256, 64)),
+                                      ("sddmm_spmm_gemm", (64, 64, 64))])
+def test_tf32_graphs_of_many_rows_go_row_first(op, sizes):
+    # the workspace tells the order: D first holds X.D, ncols x L floats
+    slnr.build()
+    for n, first in ((1 << 16, sizes[0] < 256), (1 << 17, False), (1 << 20, False)):
+        assert (csr_bytes(op, n, n, 16 * n, sizes) >= 4 * n * sizes[-1]) == first, n
