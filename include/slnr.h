@@ -213,8 +213,10 @@ slnr_status slnr_mttkrp_gemm(const slnr_csf3 *B, const float *C, const float *D,
  *   B: nrows x ncols CSR.  C, D: ncols x J.  E: J x L.  A: nrows x L (output).
  * Fused: per row i the temporary T(j) = sum_k B(i,k) C(k,j) D(k,j) (a sparse
  * row times the Hadamard product of the gathered rows) is built on chip and
- * multiplied by E at once; or (C .* D).E (ncols x L) is formed in the
- * workspace and its rows are summed, as in <SpMM,GEMM>.  Unfused: T (nrows x J) is
+ * multiplied by E at once (with C .* D, ncols x J, formed in the workspace
+ * first where many rows use each of its rows); or (C .* D).E (ncols x L) is
+ * formed in the workspace and its rows are summed, as in <SpMM,GEMM>.
+ * Unfused: T (nrows x J) is
  * written to the workspace, then A = T.E.  With allow_tf32 the T.E
  * contraction may use TF32 tensor cores. */
 slnr_status slnr_spmmh_gemm(const slnr_csr *B, const float *C, const float *D, int32_t J, const float *E,

@@ -380,12 +380,25 @@ bool premul_spmm(const slnr_csr* B, int32_t K, int32_t L, const slnr_opts* o, bo
   return premul_first(o, two ? kTwo : kOne, B->nrows, B->ncols, B->nnz, K, L, use_tc_fused(o, K, L, B->nnz));
 }
 
+// <SpMMH,GEMM> on the tensor-core row kernel: X .* X2 once per column into the
+// workspace, and one row gathered per nonzero instead of two.  The same values
+// bit for bit (the row kernel forms each product in fp32 as well).  Pays from 8
+// nonzeros a column on, in calls large enough for another launch (us, products
+// in the kernel | before it, R-MAT and uniform: 1M rows 128/128 of degree 16
+// 1742 | 1227 and 3018 | 1888, of 8 957 | 836 and 1631 | 1204, of 4 601 | 649
+// and 957 | 791; 140k 64/64 of 8 247 | 195 and 118 | 100, 32/64 109 | 101 and
+// 67 | 72).
+bool hadamard_first(const slnr_csr* B, int32_t K) {
+  return B->nnz >= 8 * (int64_t)B->ncols && B->nnz * K >= int64_t(1) << 26;
+}
+
 // (two: <SpMMH,GEMM>, two gathered matrices)
 Layout layout_spmm_gemm(const slnr_csr* B, int32_t K, int32_t L, const slnr_opts* o, bool two = false) {
   Layout l;
   if (premul_spmm(B, K, L, o, two)) return layout_premul(B->ncols, B->nnz, L, L, false);
   if (use_tc_fused(o, K, L, B->nnz)) {
     l.segs(B->nrows, B->nnz, L);
+    if (two && hadamard_first(B, K)) l.inter(sizeof(float) * (size_t)B->ncols * (size_t)K);
   } else {
     l.split(B->nrows, B->nnz, K);
     if (o->variant == SLNR_UNFUSED) l.inter(sizeof(float) * (size_t)B->nrows * (size_t)K);
@@ -1118,7 +1131,13 @@ slnr_status slnr_spmmh_gemm(const slnr_csr* B, const float* C, const float* D, i
     const SegPlan gp = seg_plan(ws, l);
     SLNR_LAUNCH("seg_count", launch_seg_count(v, gp, s));
     SLNR_LAUNCH("seg_write", launch_seg_write(v, gp, s));
-    SLNR_LAUNCH("tc_spmmh_gemm", launch_tc_spmm_gemm(J, L, v, C, E, A, gp, s, D));
+    if (hadamard_first(B, J)) {
+      float* P = reinterpret_cast<float*>(ws + l.o_inter);
+      SLNR_LAUNCH("hadamard", launch_hadamard(B->ncols, J, C, D, P, s));
+      SLNR_LAUNCH("tc_spmm_gemm", launch_tc_spmm_gemm(J, L, v, P, E, A, gp, s));
+    } else {
+      SLNR_LAUNCH("tc_spmmh_gemm", launch_tc_spmm_gemm(J, L, v, C, E, A, gp, s, D));
+    }
     SLNR_LAUNCH("combine", launch_combine(L, combine_plan(gp), nullptr, 0, A, s));
   } else if (!all_pow2(J, L)) {
     SLNR_CHECK(wide_spmm_gemm(v, C, D, J, E, L, A, ws, l, opts->variant, tc, s));

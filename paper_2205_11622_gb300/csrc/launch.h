@@ -158,6 +158,9 @@ cudaError_t launch_flat_sampled(const CsrView& B, const float* C, const float* D
 cudaError_t launch_premul(int64_t M, int K, int L, const float* X, const float* X2, const float* D, float* G,
                           cudaStream_t s);
 
+// P = X .* X2, M x K (a multiple of 4)
+cudaError_t launch_hadamard(int64_t M, int K, const float* X, const float* X2, float* P, cudaStream_t s);
+
 // rows of A (width M) that slices with nonzeros own: U(s,:) . E into row crd1[s] (U nslices x L, E L x M)
 cudaError_t launch_slices_times(const slnr_csf3& B, int L, int M, const float* U, const float* E, float* A,
                                 cudaStream_t s);

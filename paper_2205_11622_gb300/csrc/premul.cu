@@ -124,7 +124,37 @@ cudaError_t premul_width(int64_t M, int K, int L, const float* X, const float* X
   return premul_launch<64>(M, K, L, X, X2, D, G, B, s);
 }
 
+constexpr int kHadThreads = 256;
+constexpr int kHadPer = 4;  // float4s a thread has in flight of each matrix
+
+// P = X .* X2, n4 float4s: what the row kernel's Hadamard gathers would form
+// for every nonzero.  Bound by HBM: 12 bytes per value.
+__global__ void __launch_bounds__(kHadThreads) k_hadamard(int64_t n4, const float4* __restrict__ X,
+                                                          const float4* __restrict__ X2, float4* __restrict__ P) {
+  const int64_t i0 = (int64_t)blockIdx.x * (kHadThreads * kHadPer) + threadIdx.x;
+  float4 x[kHadPer], y[kHadPer];
+#pragma unroll
+  for (int k = 0; k < kHadPer; ++k) {
+    const int64_t i = i0 + k * kHadThreads;
+    x[k] = i < n4 ? __ldcs(X + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    y[k] = i < n4 ? __ldcs(X2 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+#pragma unroll
+  for (int k = 0; k < kHadPer; ++k) {
+    const int64_t i = i0 + k * kHadThreads;
+    if (i < n4) P[i] = make_float4(x[k].x * y[k].x, x[k].y * y[k].y, x[k].z * y[k].z, x[k].w * y[k].w);
+  }
+}
+
 }  // namespace
+
+cudaError_t launch_hadamard(int64_t M, int K, const float* X, const float* X2, float* P, cudaStream_t s) {
+  if (M <= 0) return cudaSuccess;
+  const int64_t n4 = M * (K / 4);
+  k_hadamard<<<SLNR_COUNTED((unsigned)ceil_div(n4, kHadThreads * kHadPer)), kHadThreads, 0, s>>>(
+      n4, reinterpret_cast<const float4*>(X), reinterpret_cast<const float4*>(X2), reinterpret_cast<float4*>(P));
+  return cudaGetLastError();
+}
 
 cudaError_t launch_premul(int64_t M, int K, int L, const float* X, const float* X2, const float* D, float* G,
                           cudaStream_t s) {

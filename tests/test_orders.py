@@ -138,3 +138,23 @@ def test_tf32_graphs_of_many_rows_go_row_first(op, sizes):
     slnr.build()
     for n, first in ((1 << 16, sizes[0] < 256), (1 << 17, False), (1 << 20, False)):
         assert (csr_bytes(op, n, n, 16 * n, sizes) >= 4 * n * sizes[-1]) == first, n
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,K,L", [(131077, 64, 64), (131073, 128, 16), (65539, 256, 32)])
+def test_hadamard_product_first_gives_the_same_bits(gpu, n, K, L):
+    # 9 nonzeros a row and one long row; the product formed here by torch and gathered by the same kernel
+    lens = np.full(n, 9)
+    lens[7] = 40000
+    w = workload("spmmh_gemm", lens.tolist(), n, K, L, 0x51A4 + n)
+    B, d = P.to_device(w)
+    got, names = phases(w, B, d, allow_tf32=True)
+    assert names == ["seg_count", "seg_write", "hadamard", "tc_spmm_gemm", "combine"]
+    assert torch.equal(got, slnr.spmm_gemm(B, d["C"] * d["D"], d["E"], allow_tf32=True))
+    # three nonzeros a column: the products in the kernel's gathers
+    few = workload("spmmh_gemm", [3] * n, n, 64, L, 0x51A4 + n)
+    B, d = P.to_device(few)
+    got, names = phases(few, B, d, allow_tf32=True)
+    if n > 1 << 17:
+        assert "tc_spmmh_gemm" in names
+        assert torch.equal(got, slnr.spmm_gemm(B, d["C"] * d["D"], d["E"], allow_tf32=True))
