@@ -190,10 +190,10 @@ slnr_status slnr_spttm_ttm(const slnr_csf3 *B, const float *C, int32_t L, const 
  * vector temporary T(i,:) (length L) stays on chip and A(i,:) = T(i,:).W
  * follows: on TF32 tensor cores with allow_tf32 when K == L in {32, 64, 128}
  * and M in {32, 64, 128}, else fp32 FFMA; or F.W (ncols x M) is formed in the
- * workspace (on TF32 tensor cores with allow_tf32 where the widths allow) and
- * each y adds a row of it to A.  Unfused: the sampled product Y (nnz values) and
- * T = Y.F (nrows x L) are written to the workspace, then A = T.W (TF32 tensor
- * cores with allow_tf32, where the widths allow). */
+ * workspace (TF32 at those widths, else fp32) and each y adds a row of it to A.
+ * Unfused: the sampled product Y (nnz values) and T = Y.F (nrows x L) are
+ * written to the workspace, then A = T.W (TF32 tensor cores with allow_tf32,
+ * where the widths allow). */
 slnr_status slnr_sddmm_spmm_gemm(const slnr_csr *B, const float *C, const float *D, int32_t K, const float *F,
                                  int32_t L, const float *W, int32_t M, float *A, const slnr_opts *opts);
 

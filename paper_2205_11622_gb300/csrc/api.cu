@@ -330,9 +330,9 @@ bool use_tc_fused(const slnr_opts* o, int32_t K, int32_t L, int64_t nnz) {
 //    100k: 56 | 37, 70 | 110), 64k at K = 32 (50k R-MAT 83 | 60), 128k at
 //    K >= 64, from 64k on at K >= 128 of degrees of 8 or more.  Two gathered
 //    matrices or sampled rows move the line up to 128k throughout.
-bool use_tc_premul(const slnr_opts* o, int32_t K, int32_t L, int64_t nnz) {
-  return o->allow_tf32 != 0 && tc_split_supported(K, L) && nnz >= kTcFusedMinNnz;
-}
+// The product itself rounds to tf32 only in calls whose row kernel does: the
+// others keep fp32 throughout.
+bool premul_tc(bool row_tc, int32_t K, int32_t L) { return row_tc && tc_split_supported(K, L); }
 enum PremulKind { kOne, kTwo, kSampledRows, kFibers };
 
 // Whether the two orders give nearly the same values where the row kernel runs
@@ -832,7 +832,7 @@ slnr_status slnr_spmm_gemm(const slnr_csr* B, const float* C, int32_t K, const f
   if (B->nrows == 0) return SLNR_OK;
   cudaStream_t s = static_cast<cudaStream_t>(opts->stream);
   char* ws = static_cast<char*>(opts->workspace);
-  const bool pre = premul_spmm(B, K, L, opts, false), pre_tc = use_tc_premul(opts, K, L, B->nnz);
+  const bool pre = premul_spmm(B, K, L, opts, false), pre_tc = premul_tc(use_tc_fused(opts, K, L, B->nnz), K, L);
   SLNR_CHECK(begin(ws, s, opts->validate != 0,
                    [&](WsHeader* h) { return launch_validate_csr(*B, h, s); }, pre && !pre_tc));
   const CsrView v = csr_view(B);
@@ -930,7 +930,7 @@ slnr_status slnr_spttm_ttm(const slnr_csf3* B, const float* C, int32_t L, const 
   SLNR_CHECK(check_ws(opts, l.total()));
   cudaStream_t s = static_cast<cudaStream_t>(opts->stream);
   char* ws = static_cast<char*>(opts->workspace);
-  const bool pre = premul_spttm(B, L, M, opts), pre_tc = use_tc_premul(opts, L, M, B->nnz);
+  const bool pre = premul_spttm(B, L, M, opts), pre_tc = premul_tc(use_tc_fused(opts, L, M, B->nnz), L, M);
   SLNR_CHECK(begin(ws, s, opts->validate != 0,
                    [&](WsHeader* h) { return launch_validate_csf(*B, h, s); }, pre && !pre_tc));
   // A's two compressed levels are B's (the (i,j) pattern is unchanged)
@@ -987,7 +987,8 @@ slnr_status slnr_sddmm_spmm_gemm(const slnr_csr* B, const float* C, const float*
   if (B->nrows == 0) return SLNR_OK;
   cudaStream_t s = static_cast<cudaStream_t>(opts->stream);
   char* ws = static_cast<char*>(opts->workspace);
-  const bool pre = premul_sampled(B, K, L, M, opts), pre_tc = use_tc_premul(opts, L, M, B->nnz);
+  const bool pre = premul_sampled(B, K, L, M, opts),
+             pre_tc = premul_tc(use_tc_sampled(opts, K, L, M, B->nnz), L, M);
   SLNR_CHECK(begin(ws, s, opts->validate != 0,
                    [&](WsHeader* h) { return launch_validate_csr(*B, h, s); }, pre && !pre_tc));
   const CsrView v = csr_view(B);
@@ -1118,7 +1119,7 @@ slnr_status slnr_spmmh_gemm(const slnr_csr* B, const float* C, const float* D, i
   if (B->nrows == 0) return SLNR_OK;
   cudaStream_t s = static_cast<cudaStream_t>(opts->stream);
   char* ws = static_cast<char*>(opts->workspace);
-  const bool pre = premul_spmm(B, J, L, opts, true), pre_tc = use_tc_premul(opts, J, L, B->nnz);
+  const bool pre = premul_spmm(B, J, L, opts, true), pre_tc = premul_tc(use_tc_fused(opts, J, L, B->nnz), J, L);
   SLNR_CHECK(begin(ws, s, opts->validate != 0,
                    [&](WsHeader* h) { return launch_validate_csr(*B, h, s); }, pre && !pre_tc));
   const CsrView v = csr_view(B);

@@ -158,3 +158,17 @@ def test_hadamard_product_first_gives_the_same_bits(gpu, n, K, L):
     if n > 1 << 17:
         assert "tc_spmmh_gemm" in names
         assert torch.equal(got, slnr.spmm_gemm(B, d["C"] * d["D"], d["E"], allow_tf32=True))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("K,L,M", [(32, 64, 64), (16, 16, 16), (64, 64, 16), (128, 64, 128), (100, 64, 64)])
+def test_sampled_gemm_stays_fp32_at_widths_without_a_tensor_core_kernel(gpu, K, L, M):
+    # TF32 allowed or not: the same bits.  36000 nonzeros: past the size from which the tensor cores are taken
+    n = 3000
+    B = csr_of([12] * n, n, 0x51A4 + K)
+    r = wl.Rng(K + L + M)
+    w = wl.Workload("sampled", "sddmm_spmm_gemm", B, {"C": wl.normal(r, (n, K)), "D": wl.normal(r, (n, K)),
+                                                      "F": wl.normal(r, (n, L)), "W": wl.normal(r, (L, M))},
+                    {"K": K, "L": L, "M": M})
+    dB, d = P.to_device(w)
+    assert torch.equal(phases(w, dB, d, allow_tf32=True)[0], phases(w, dB, d, allow_tf32=False)[0])
