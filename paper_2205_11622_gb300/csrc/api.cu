@@ -353,11 +353,30 @@ bool premul_near(PremulKind kind, int64_t nrows, int64_t ncols, int64_t nnz, int
   return nrows < (rounded ? 128 : 64) * 1024;
 }
 
+// Whether the columns that X has more than B has rows are worth their share of
+// the product: D first forms K L products for each of them, row first for the
+// rows only.  In units of one gathered value (4 bytes at 10 TB/s): a column of
+// the fp32 product K L / 4 + 2 L, of the tensor cores' 3 (K + L) (it is bound by
+// memory); against the narrower gathers, a quarter of row first's gathers, and
+// 2^25 for its inspector and the chunks of heavy rows.  Measured on 788 shapes
+// of 500 to 200k rows, up to 128 times as many columns, 2 to 768 nonzeros a row
+// (uniform and skewed), widths 16 to 256: D first on 469 of them, 0.99 to 7.4
+// times as fast as row first (median 1.6); of the others down to 0.07 (32k x
+// 4M, 4M nonzeros, 256/256 845 us | 13006).
+bool premul_columns_pay(PremulKind kind, int64_t nrows, int64_t ncols, int64_t nnz, int32_t K, int32_t L, bool row_tc) {
+  if (ncols <= nrows) return true;
+  const int64_t gathered = kind == kTwo ? 2 * K : K;
+  const int64_t column = premul_tc(row_tc, K, L) ? 3 * (gathered + L) : K * L / 4 + 2 * L;
+  const int64_t narrower = gathered > L ? gathered - L : 0;
+  return (ncols - nrows) * column <= nnz * (narrower + K / 4) + (int64_t(1) << 25);
+}
+
 bool premul_first(const slnr_opts* o, PremulKind kind, int64_t nrows, int64_t ncols, int64_t nnz, int32_t K, int32_t L,
                   bool row_tc) {
   if (o->variant != SLNR_FUSED || nnz < 1 || nnz < ncols) return false;
   if (L > K && nnz > 64 * nrows) return false;  // long rows: the narrower rows are gathered
   if (row_tc && !premul_near(kind, nrows, ncols, nnz, K, L)) return false;
+  if (!premul_columns_pay(kind, nrows, ncols, nnz, K, L, row_tc)) return false;
   const int64_t k = 1024;
   if (kind == kFibers) return !row_tc || L <= 2 * K || nnz < 2048 * k;
   if (kind == kSampledRows && L > 2 * K && nrows >= (L > 4 * K ? 0 : 64 * k)) return false;

@@ -94,6 +94,7 @@ def test_premultiplied_sums(slnr, op, J, L, kind):
     lens = structure(kind, rng)
     ncols = {"empty_runs": 45, "window_ends": 2000, "long": 9100}[kind]
     lens = [min(n, ncols) for n in lens]
+    lens += [0] * (ncols - len(lens))  # as many rows as columns: the calls that take the product first
     B = csr(lens, ncols, rng, 0x51A4 + J)
     r = wl.Rng(0x51A4 + 7 * L)
     names = ("C", "D") if op == "spmm_gemm" else ("C", "D", "E")
@@ -169,7 +170,9 @@ def columns_workload(ncols, K, L, two, positive=False):
     r = wl.Rng(0x51A4 + ncols + K + L)
     crd = np.concatenate([np.sort(np.random.default_rng(i).choice(ncols, per, replace=False)) for i in range(n)])
     lo = 0.5 if positive else -1
-    B = wl.CSR(n, ncols, np.arange(n + 1, dtype=np.int32) * per, crd.astype(np.int32), wl.uniform(r, per * n, lo, 1))
+    # as many rows as columns (the others empty): the calls that take the product first
+    pos = np.minimum(np.arange(max(n, ncols) + 1), n).astype(np.int32) * per
+    B = wl.CSR(len(pos) - 1, ncols, pos, crd.astype(np.int32), wl.uniform(r, per * n, lo, 1))
     X, X2 = wl.uniform(r, (ncols, K), lo, 1), wl.uniform(r, (ncols, K), lo, 1)
     D = np.round(wl.uniform(r, (K, L), lo, 1) * 512).astype(np.float32) / 512
     if two:
@@ -180,13 +183,19 @@ def columns_workload(ncols, K, L, two, positive=False):
 @pytest.mark.gpu
 @pytest.mark.parametrize("two", [False, True])
 @pytest.mark.parametrize("ncols,K,L", [(1, 16, 16), (127, 128, 128), (128, 32, 64), (129, 128, 16), (8 * 30 + 1, 16, 32),
-                                       (130000, 128, 128), (40000, 64, 64), (19457, 32, 16)])
+                                       (65000, 128, 128), (40000, 64, 64), (19457, 32, 16)])
 def test_split_product_rows(slnr, ncols, K, L, two):
     # one tile, its edges, one tile more than a CTA each, several tiles per CTA; the bound is the one above
     w = columns_workload(ncols, K, L, two)
     ref, ref_abs = oracle.get().run(w)
     dB, dd = P.to_device(w)
-    out = slnr.run(w.op, dB, dd, allow_tf32=True)
+    slnr.timing_enable(True)
+    try:
+        out = slnr.run(w.op, dB, dd, allow_tf32=True)
+        names = [n for n, _ in slnr.timing_read()]
+    finally:
+        slnr.timing_enable(False)
+    assert names[0] == "tc_premul", names
     assert P.rel_err(out.cpu().numpy(), ref, ref_abs) <= 1e-5
 
 

@@ -124,8 +124,14 @@ def test_tf32_values_stay_where_rows_are_long(gpu, op, K, L):
 
 
 def csr_bytes(op, nrows, ncols, nnz, sizes, tf32=1):
+    """Workspace of the fused call; fibers for spttm_ttm (50 to a slice)."""
     n = ctypes.c_size_t(0)
-    B = slnr.slnr_csr(nrows, ncols, nnz, 0x1000, 0x2000, 0x3000)
+    if op == "spttm_ttm":
+        B = slnr.slnr_csf3()
+        B.dim[0], B.dim[1], B.dim[2] = -(-nrows // 50), 50, ncols
+        B.nnz, B.nslices, B.nfibers = nnz, B.dim[0], nrows
+    else:
+        B = slnr.slnr_csr(nrows, ncols, nnz, 0x1000, 0x2000, 0x3000)
     o = slnr.slnr_opts(0, tf32, 0, 0, None, None, 0)
     assert getattr(slnr.lib(), f"slnr_{op}_workspace")(ctypes.byref(B), *sizes, ctypes.byref(o), ctypes.byref(n)) == 0
     return n.value
@@ -172,3 +178,19 @@ def test_sampled_gemm_stays_fp32_at_widths_without_a_tensor_core_kernel(gpu, K, 
                     {"K": K, "L": L, "M": M})
     dB, d = P.to_device(w)
     assert torch.equal(phases(w, dB, d, allow_tf32=True)[0], phases(w, dB, d, allow_tf32=False)[0])
+
+
+@pytest.mark.parametrize("op,nrows,ncols,nnz,sizes,tf32,first", [
+    ("spmm_gemm", 4096, 1 << 20, 1 << 20, (256, 256), 0, False),      # 137 GFLOP for 4096 rows
+    ("spmm_gemm", 4096, 1 << 20, 1 << 20, (128, 128), 1, False),
+    ("spmm_gemm", 1000, 1000000, 1000000, (64, 64), 0, False),
+    ("spmmh_gemm", 4096, 1 << 20, 1 << 20, (128, 128), 1, False),
+    ("sddmm_spmm_gemm", 1000, 1000000, 1000000, (1024, 1024, 1024), 0, False),
+    ("spttm_ttm", 4096, 1 << 20, 1 << 20, (128, 128), 0, False),      # a long third mode
+    ("spmm_gemm", 4096, 16384, 16384 * 8, (64, 64), 0, True),         # few columns more: the sums pay for them
+    ("spmm_gemm", 150001, 150001, 2400016, (64, 32), 0, True),
+    ("spttm_ttm", 2500000, 5000, 20000000, (64, 64), 0, True),
+])
+def test_many_columns_go_row_first(op, nrows, ncols, nnz, sizes, tf32, first):
+    slnr.build()
+    assert (csr_bytes(op, nrows, ncols, nnz, sizes, tf32) >= 4 * ncols * sizes[-1]) == first
