@@ -120,6 +120,8 @@ typedef struct slnr_opts {
  * Bytes of workspace the matching call needs for these sizes and options
  * (variant changes it).  Depends only on the sizes and counts in the
  * structure descriptor, never on device data.  Pointers in B may be NULL.
+ * Where the call would take a product of the dense matrices first, a smaller
+ * workspace that holds the row-by-row schedule is accepted too and gets that.
  * Returns SLNR_OK and writes *bytes, or an argument error. */
 slnr_status slnr_spmm_gemm_workspace(const slnr_csr *B, int32_t K, int32_t L, const slnr_opts *opts,
                                      size_t *bytes);

@@ -15,6 +15,7 @@ ctypes structures and raw device pointers; the snake-case wrappers
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 import threading
 from dataclasses import dataclass
@@ -310,7 +311,6 @@ def device_flags(workspace=None) -> int:
 
 
 _VARIANTS = {"fused": FUSED, "unfused": UNFUSED, FUSED: FUSED, UNFUSED: UNFUSED}
-_ERR_WORKSPACE = 4
 
 
 def _stream_ptr(stream) -> int:
@@ -321,14 +321,36 @@ def _stream_ptr(stream) -> int:
     return c._cuda_getCurrentRawStream(c._cuda_getDevice())
 
 
-def _run(name, B, args, sizes, variant, allow_tf32, validate, workspace, stream):
-    """Call entry point `name` with the structure B, `args` and the options.
+@functools.lru_cache(maxsize=4096)
+def _ws_bytes(name, shape, sizes, variant, tf32) -> int:
+    """Workspace of entry point `name`: a function of the sizes and options alone."""
+    if len(shape) == 3:
+        B = slnr_csr(*shape, None, None, None)
+    else:
+        B = slnr_csf3((ctypes.c_int32 * 3)(*shape[:3]), *shape[3:])
+    o = slnr_opts(variant, tf32, 0, 0, None, None, 0)
+    return _query(name + "_workspace", ctypes.byref(B), *sizes, ctypes.byref(o))
 
-    The workspace that is there is tried first: the library checks its size
-    before it enqueues anything and says SLNR_ERR_WORKSPACE if it is too small;
-    only then is the size asked for (with `sizes`) and the buffer grown.  Small
-    calls are bound by this function, not by their kernels.
-    """
+
+def _room(workspace, need):
+    """(buffer of `need` bytes, None), or where the device has no room for that (the largest half of it, half of
+    that, ... that it has room for, the error): some calls run in less."""
+    oom = _torch().OutOfMemoryError
+    try:
+        return workspace.get(need), None
+    except oom as e:
+        short = e
+    while need > 256:
+        need //= 2
+        try:
+            return workspace.get(need), short
+        except oom:
+            pass
+    raise short
+
+
+def _run(name, B, args, sizes, variant, allow_tf32, validate, workspace, stream):
+    """Call entry point `name` with the structure B, `args` and the options."""
     L = _lib if _lib is not None else lib()
     s = _stream_ptr(stream)
     if workspace is None:
@@ -337,20 +359,18 @@ def _run(name, B, args, sizes, variant, allow_tf32, validate, workspace, stream)
         if workspace is None:
             workspace = _default_ws.setdefault((dev, s), Workspace(device=f"cuda:{dev}"))
     v = _VARIANTS.get(variant)
-    o = slnr_opts(int(variant) if v is None else v, 1 if allow_tf32 else 0, 1 if validate else 0, 0, s, None, 0)
-    bs, os_ = ctypes.byref(B), ctypes.byref(o)
-    status = _ERR_WORKSPACE
-    buf = workspace.buf
-    if buf is not None:
-        o.workspace, o.workspace_bytes = buf.data_ptr(), buf.numel()
-        status = getattr(L, name)(bs, *args, os_)
-    if status == _ERR_WORKSPACE:
-        buf = workspace.get(_query(name + "_workspace", bs, *sizes, os_))
-        o.workspace, o.workspace_bytes = buf.data_ptr(), buf.numel()
-        status = getattr(L, name)(bs, *args, os_)
+    v = int(variant) if v is None else v
+    tf32 = 1 if allow_tf32 else 0
+    shape = (B.nrows, B.ncols, B.nnz) if type(B) is slnr_csr else (*B.dim, B.nnz, B.nslices, B.nfibers)
+    need, buf, short = _ws_bytes(name, shape, sizes, v, tf32), workspace.buf, None
+    if buf is None or buf.numel() < need:
+        buf, short = _room(workspace, need)
+    o = slnr_opts(v, tf32, 1 if validate else 0, 0, s, buf.data_ptr(), buf.numel())
     _last_ws[0] = buf
+    status = getattr(L, name)(ctypes.byref(B), *args, ctypes.byref(o))
     if status != 0:
-        raise SlnrError(status, name, last_error())
+        raise short if short is not None and STATUS[status] == "SLNR_ERR_WORKSPACE" else \
+            SlnrError(status, name, last_error())
 
 
 def _dense(x, name):

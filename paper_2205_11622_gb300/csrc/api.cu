@@ -395,10 +395,6 @@ Layout layout_premul(int64_t ncols, int64_t nnz, int wm, int32_t L, bool sampled
   return l;
 }
 
-bool premul_spmm(const slnr_csr* B, int32_t K, int32_t L, const slnr_opts* o, bool two) {
-  return premul_first(o, two ? kTwo : kOne, B->nrows, B->ncols, B->nnz, K, L, use_tc_fused(o, K, L, B->nnz));
-}
-
 // <SpMMH,GEMM> on the tensor-core row kernel: X .* X2 once per column into the
 // workspace, and one row gathered per nonzero instead of two.  The same values
 // bit for bit (the row kernel forms each product in fp32 as well).  Pays from 8
@@ -411,13 +407,38 @@ bool hadamard_first(const slnr_csr* B, int32_t K) {
   return B->nnz >= 8 * (int64_t)B->ncols && B->nnz * K >= int64_t(1) << 26;
 }
 
+// The order that a call takes, and its workspace: kProductFirst and
+// kHadamardFirst hold a row per column there.
+enum Order { kRowFirst, kHadamardFirst, kProductFirst };
+
+// The layout of the order that the call prefers (what the workspace query
+// reports), or, if a smaller workspace holds row first, of that.
+template <typename LayoutOf>
+Layout fit(const slnr_opts* o, Order& order, LayoutOf layout_of) {
+  const Layout l = layout_of(order);
+  if (order != kRowFirst && l.total() > o->workspace_bytes) {
+    const Layout rows = layout_of(kRowFirst);
+    if (rows.total() <= o->workspace_bytes) {
+      order = kRowFirst;
+      return rows;
+    }
+  }
+  return l;
+}
+
 // (two: <SpMMH,GEMM>, two gathered matrices)
-Layout layout_spmm_gemm(const slnr_csr* B, int32_t K, int32_t L, const slnr_opts* o, bool two = false) {
+Order order_spmm_gemm(const slnr_csr* B, int32_t K, int32_t L, const slnr_opts* o, bool two) {
+  const bool row_tc = use_tc_fused(o, K, L, B->nnz);
+  if (premul_first(o, two ? kTwo : kOne, B->nrows, B->ncols, B->nnz, K, L, row_tc)) return kProductFirst;
+  return two && row_tc && hadamard_first(B, K) ? kHadamardFirst : kRowFirst;
+}
+
+Layout layout_spmm_gemm(const slnr_csr* B, int32_t K, int32_t L, const slnr_opts* o, Order order) {
   Layout l;
-  if (premul_spmm(B, K, L, o, two)) return layout_premul(B->ncols, B->nnz, L, L, false);
+  if (order == kProductFirst) return layout_premul(B->ncols, B->nnz, L, L, false);
   if (use_tc_fused(o, K, L, B->nnz)) {
     l.segs(B->nrows, B->nnz, L);
-    if (two && hadamard_first(B, K)) l.inter(sizeof(float) * (size_t)B->ncols * (size_t)K);
+    if (order == kHadamardFirst) l.inter(sizeof(float) * (size_t)B->ncols * (size_t)K);
   } else {
     l.split(B->nrows, B->nnz, K);
     if (o->variant == SLNR_UNFUSED) l.inter(sizeof(float) * (size_t)B->nrows * (size_t)K);
@@ -469,13 +490,14 @@ Layout layout_mttkrp(const slnr_csf3* B, int32_t L, int variant) {
   return l;
 }
 
-bool premul_spttm(const slnr_csf3* B, int32_t L, int32_t M, const slnr_opts* o) {
-  return premul_first(o, kFibers, B->nfibers, B->dim[2], B->nnz, L, M, use_tc_fused(o, L, M, B->nnz));
+Order order_spttm_ttm(const slnr_csf3* B, int32_t L, int32_t M, const slnr_opts* o) {
+  return premul_first(o, kFibers, B->nfibers, B->dim[2], B->nnz, L, M, use_tc_fused(o, L, M, B->nnz)) ? kProductFirst
+                                                                                                    : kRowFirst;
 }
 
-Layout layout_spttm_ttm(const slnr_csf3* B, int32_t L, int32_t M, const slnr_opts* o) {
+Layout layout_spttm_ttm(const slnr_csf3* B, int32_t L, int32_t M, const slnr_opts* o, Order order) {
   Layout l;
-  if (premul_spttm(B, L, M, o)) return layout_premul(B->dim[2], B->nnz, M, M, false);
+  if (order == kProductFirst) return layout_premul(B->dim[2], B->nnz, M, M, false);
   if (use_tc_fused(o, L, M, B->nnz)) {
     l.segs(B->nfibers, B->nnz, M);
   } else {
@@ -491,15 +513,16 @@ bool use_tc_sampled(const slnr_opts* o, int32_t K, int32_t L, int32_t M, int64_t
   return o->variant == SLNR_FUSED && o->allow_tf32 != 0 && tc_sampled_supported(K, L, M) && nnz >= kTcFusedMinNnz;
 }
 
-bool premul_sampled(const slnr_csr* B, int32_t K, int32_t L, int32_t M, const slnr_opts* o) {
-  return premul_first(o, kSampledRows, B->nrows, B->ncols, B->nnz, L, M, use_tc_sampled(o, K, L, M, B->nnz));
+Order order_sddmm_spmm_gemm(const slnr_csr* B, int32_t K, int32_t L, int32_t M, const slnr_opts* o) {
+  return premul_first(o, kSampledRows, B->nrows, B->ncols, B->nnz, L, M, use_tc_sampled(o, K, L, M, B->nnz))
+             ? kProductFirst
+             : kRowFirst;
 }
 
-Layout layout_sddmm_spmm_gemm(const slnr_csr* B, int32_t K, int32_t L, int32_t M, const slnr_opts* o) {
+Layout layout_sddmm_spmm_gemm(const slnr_csr* B, int32_t K, int32_t L, int32_t M, const slnr_opts* o, Order order) {
   const int variant = o->variant;
   Layout l;
-  if (premul_sampled(B, K, L, M, o))
-    return layout_premul(B->ncols, B->nnz, K > M ? K : M, M, true);
+  if (order == kProductFirst) return layout_premul(B->ncols, B->nnz, K > M ? K : M, M, true);
   if (use_tc_sampled(o, K, L, M, B->nnz)) {
     l.segs(B->nrows, B->nnz, M);
     return l;
@@ -766,7 +789,7 @@ slnr_status slnr_spmm_gemm_workspace(const slnr_csr* B, int32_t K, int32_t L, co
   SLNR_CHECK(check_dims("K", K));
   SLNR_CHECK(check_dims("L", L));
   if (!bytes) return fail(SLNR_ERR_NULL, "bytes is NULL");
-  *bytes = layout_spmm_gemm(B, K, L, opts).total();
+  *bytes = layout_spmm_gemm(B, K, L, opts, order_spmm_gemm(B, K, L, opts, false)).total();
   return SLNR_OK;
 }
 
@@ -797,7 +820,7 @@ slnr_status slnr_spttm_ttm_workspace(const slnr_csf3* B, int32_t L, int32_t M, c
   SLNR_CHECK(check_dims("L", L));
   SLNR_CHECK(check_dims("M", M));
   if (!bytes) return fail(SLNR_ERR_NULL, "bytes is NULL");
-  *bytes = layout_spttm_ttm(B, L, M, opts).total();
+  *bytes = layout_spttm_ttm(B, L, M, opts, order_spttm_ttm(B, L, M, opts)).total();
   return SLNR_OK;
 }
 
@@ -809,7 +832,7 @@ slnr_status slnr_sddmm_spmm_gemm_workspace(const slnr_csr* B, int32_t K, int32_t
   SLNR_CHECK(check_dims("L", L));
   SLNR_CHECK(check_dims("M", M));
   if (!bytes) return fail(SLNR_ERR_NULL, "bytes is NULL");
-  *bytes = layout_sddmm_spmm_gemm(B, K, L, M, opts).total();
+  *bytes = layout_sddmm_spmm_gemm(B, K, L, M, opts, order_sddmm_spmm_gemm(B, K, L, M, opts)).total();
   return SLNR_OK;
 }
 
@@ -831,7 +854,7 @@ slnr_status slnr_spmmh_gemm_workspace(const slnr_csr* B, int32_t J, int32_t L, c
   SLNR_CHECK(check_dims("J", J));
   SLNR_CHECK(check_dims("L", L));
   if (!bytes) return fail(SLNR_ERR_NULL, "bytes is NULL");
-  *bytes = layout_spmm_gemm(B, J, L, opts, true).total();
+  *bytes = layout_spmm_gemm(B, J, L, opts, order_spmm_gemm(B, J, L, opts, true)).total();
   return SLNR_OK;
 }
 
@@ -846,12 +869,13 @@ slnr_status slnr_spmm_gemm(const slnr_csr* B, const float* C, int32_t K, const f
   SLNR_CHECK(check_dense("C", C));
   SLNR_CHECK(check_dense("D", D));
   SLNR_CHECK(check_dense("A", A));
-  const Layout l = layout_spmm_gemm(B, K, L, opts);
+  Order order = order_spmm_gemm(B, K, L, opts, false);
+  const Layout l = fit(opts, order, [&](Order x) { return layout_spmm_gemm(B, K, L, opts, x); });
   SLNR_CHECK(check_ws(opts, l.total()));
   if (B->nrows == 0) return SLNR_OK;
   cudaStream_t s = static_cast<cudaStream_t>(opts->stream);
   char* ws = static_cast<char*>(opts->workspace);
-  const bool pre = premul_spmm(B, K, L, opts, false), pre_tc = premul_tc(use_tc_fused(opts, K, L, B->nnz), K, L);
+  const bool pre = order == kProductFirst, pre_tc = premul_tc(use_tc_fused(opts, K, L, B->nnz), K, L);
   SLNR_CHECK(begin(ws, s, opts->validate != 0,
                    [&](WsHeader* h) { return launch_validate_csr(*B, h, s); }, pre && !pre_tc));
   const CsrView v = csr_view(B);
@@ -945,11 +969,12 @@ slnr_status slnr_spttm_ttm(const slnr_csf3* B, const float* C, int32_t L, const 
   if (!A_pos1 || !A_pos2 || (B->nslices > 0 && !A_crd1) || (B->nfibers > 0 && !A_crd2))
     return fail(SLNR_ERR_NULL, "an output index array of A is NULL");
   if (B->nfibers > 0) SLNR_CHECK(check_dense("A_vals", A_vals));
-  const Layout l = layout_spttm_ttm(B, L, M, opts);
+  Order order = order_spttm_ttm(B, L, M, opts);
+  const Layout l = fit(opts, order, [&](Order x) { return layout_spttm_ttm(B, L, M, opts, x); });
   SLNR_CHECK(check_ws(opts, l.total()));
   cudaStream_t s = static_cast<cudaStream_t>(opts->stream);
   char* ws = static_cast<char*>(opts->workspace);
-  const bool pre = premul_spttm(B, L, M, opts), pre_tc = premul_tc(use_tc_fused(opts, L, M, B->nnz), L, M);
+  const bool pre = order == kProductFirst, pre_tc = premul_tc(use_tc_fused(opts, L, M, B->nnz), L, M);
   SLNR_CHECK(begin(ws, s, opts->validate != 0,
                    [&](WsHeader* h) { return launch_validate_csf(*B, h, s); }, pre && !pre_tc));
   // A's two compressed levels are B's (the (i,j) pattern is unchanged)
@@ -1001,12 +1026,13 @@ slnr_status slnr_sddmm_spmm_gemm(const slnr_csr* B, const float* C, const float*
   SLNR_CHECK(check_dense("F", F));
   SLNR_CHECK(check_dense("W", W));
   SLNR_CHECK(check_dense("A", A));
-  const Layout l = layout_sddmm_spmm_gemm(B, K, L, M, opts);
+  Order order = order_sddmm_spmm_gemm(B, K, L, M, opts);
+  const Layout l = fit(opts, order, [&](Order x) { return layout_sddmm_spmm_gemm(B, K, L, M, opts, x); });
   SLNR_CHECK(check_ws(opts, l.total()));
   if (B->nrows == 0) return SLNR_OK;
   cudaStream_t s = static_cast<cudaStream_t>(opts->stream);
   char* ws = static_cast<char*>(opts->workspace);
-  const bool pre = premul_sampled(B, K, L, M, opts),
+  const bool pre = order == kProductFirst,
              pre_tc = premul_tc(use_tc_sampled(opts, K, L, M, B->nnz), L, M);
   SLNR_CHECK(begin(ws, s, opts->validate != 0,
                    [&](WsHeader* h) { return launch_validate_csr(*B, h, s); }, pre && !pre_tc));
@@ -1133,12 +1159,13 @@ slnr_status slnr_spmmh_gemm(const slnr_csr* B, const float* C, const float* D, i
   SLNR_CHECK(check_dense("D", D));
   SLNR_CHECK(check_dense("E", E));
   SLNR_CHECK(check_dense("A", A));
-  const Layout l = layout_spmm_gemm(B, J, L, opts, true);
+  Order order = order_spmm_gemm(B, J, L, opts, true);
+  const Layout l = fit(opts, order, [&](Order x) { return layout_spmm_gemm(B, J, L, opts, x); });
   SLNR_CHECK(check_ws(opts, l.total()));
   if (B->nrows == 0) return SLNR_OK;
   cudaStream_t s = static_cast<cudaStream_t>(opts->stream);
   char* ws = static_cast<char*>(opts->workspace);
-  const bool pre = premul_spmm(B, J, L, opts, true), pre_tc = premul_tc(use_tc_fused(opts, J, L, B->nnz), J, L);
+  const bool pre = order == kProductFirst, pre_tc = premul_tc(use_tc_fused(opts, J, L, B->nnz), J, L);
   SLNR_CHECK(begin(ws, s, opts->validate != 0,
                    [&](WsHeader* h) { return launch_validate_csr(*B, h, s); }, pre && !pre_tc));
   const CsrView v = csr_view(B);
@@ -1151,7 +1178,7 @@ slnr_status slnr_spmmh_gemm(const slnr_csr* B, const float* C, const float* D, i
     const SegPlan gp = seg_plan(ws, l);
     SLNR_LAUNCH("seg_count", launch_seg_count(v, gp, s));
     SLNR_LAUNCH("seg_write", launch_seg_write(v, gp, s));
-    if (hadamard_first(B, J)) {
+    if (order == kHadamardFirst) {
       float* P = reinterpret_cast<float*>(ws + l.o_inter);
       SLNR_LAUNCH("hadamard", launch_hadamard(B->ncols, J, C, D, P, s));
       SLNR_LAUNCH("tc_spmm_gemm", launch_tc_spmm_gemm(J, L, v, P, E, A, gp, s));

@@ -194,3 +194,45 @@ def test_sampled_gemm_stays_fp32_at_widths_without_a_tensor_core_kernel(gpu, K, 
 def test_many_columns_go_row_first(op, nrows, ncols, nnz, sizes, tf32, first):
     slnr.build()
     assert (csr_bytes(op, nrows, ncols, nnz, sizes, tf32) >= 4 * ncols * sizes[-1]) == first
+
+
+class Scarce(slnr.Workspace):
+    """A device with room for `most` bytes of workspace."""
+
+    def __init__(self, most):
+        super().__init__()
+        self.most = most
+
+    def get(self, nbytes):
+        if nbytes > self.most:
+            raise torch.OutOfMemoryError("no room")
+        return super().get(nbytes)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("op,K,L,row_kernel", [("spmm_gemm", 64, 64, "tc_spmm_gemm"), ("spmm_gemm", 100, 48, "w_spmm_gemm_tiles"),
+                                               ("spmmh_gemm", 64, 64, "tc_spmmh_gemm"),
+                                               ("sddmm_spmm_gemm", 64, 64, "tc_sddmm_spmm_gemm"),
+                                               ("spttm_ttm", 64, 64, "tc_spmm_gemm")])
+def test_a_workspace_that_holds_row_first_is_enough(gpu, op, K, L, row_kernel):
+    n = 20000
+    w = workload(op, [5] * n, n if op != "spttm_ttm" else 1000, K, L, 0x51A4 + K)
+    B, d = P.to_device(w)
+    ref, ref_abs = oracle.get().run(w)
+    own = slnr.Workspace()
+    small = workload(op, [5] * 100, n if op != "spttm_ttm" else 1000, K, L, 1)
+    phases(small, *P.to_device(small), workspace=own)
+    full, names = phases(w, B, d, workspace=own)  # a small call's workspace before it: the order is the same
+    assert names[-1].startswith("flat_"), names
+    rows, names = phases(w, B, d, workspace=Scarce(own.buf.numel() // 2))
+    assert row_kernel in names, names
+    for got in (full, rows):
+        assert P.rel_err(got.cpu().numpy(), ref, ref_abs) <= P.TOL_TF32
+    with pytest.raises(torch.OutOfMemoryError):  # not enough for either
+        slnr.run(op, B, d, workspace=Scarce(4096))
+    few = torch.empty(4096, dtype=torch.uint8, device="cuda")
+    ws = slnr.Workspace()
+    ws.buf, ws.get = few, lambda n: few
+    with pytest.raises(slnr.SlnrError) as e:
+        slnr.run(op, B, d, workspace=ws)
+    assert e.value.status == 4
