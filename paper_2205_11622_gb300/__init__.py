@@ -317,8 +317,10 @@ def _stream_ptr(stream) -> int:
     """The cudaStream_t of a torch stream (None: the current device's current stream)."""
     if stream is not None:
         return stream.cuda_stream
-    c = _torch()._C
-    return c._cuda_getCurrentRawStream(c._cuda_getDevice())
+    torch = _torch()
+    # without the stream object that current_stream() makes, where this torch has that accessor (calls take 20 us)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return torch.cuda.current_stream().cuda_stream if raw is None else raw(torch.cuda.current_device())
 
 
 @functools.lru_cache(maxsize=4096)
@@ -354,7 +356,7 @@ def _run(name, B, args, sizes, variant, allow_tf32, validate, workspace, stream)
     L = _lib if _lib is not None else lib()
     s = _stream_ptr(stream)
     if workspace is None:
-        dev = _torch()._C._cuda_getDevice()
+        dev = _torch().cuda.current_device()
         workspace = _default_ws.get((dev, s))
         if workspace is None:
             workspace = _default_ws.setdefault((dev, s), Workspace(device=f"cuda:{dev}"))

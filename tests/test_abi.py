@@ -117,3 +117,14 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(slnr, "LIBRARY", str(tmp_path / "nope.so"))
     with pytest.raises(RuntimeError, match="not built"):
         slnr.lib()
+
+
+@pytest.mark.parametrize("raw", [True, False])
+def test_stream_lookup_needs_no_private_name(monkeypatch, raw):
+    # torch's raw accessor is used where it exists; the public functions do otherwise
+    from types import SimpleNamespace as NS
+    cuda = NS(current_device=lambda: 3, current_stream=lambda: NS(cuda_stream=0x700))
+    c = NS(_cuda_getCurrentRawStream=lambda dev: 0x700 if dev == 3 else None) if raw else NS()
+    monkeypatch.setattr(slnr, "_torch", lambda: NS(_C=c, cuda=cuda))
+    assert slnr._stream_ptr(None) == 0x700
+    assert slnr._stream_ptr(NS(cuda_stream=0x900)) == 0x900
