@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "range.h"
 #include "slnr.h"
 
 namespace slnr {
@@ -147,7 +148,7 @@ __device__ __forceinline__ void gather_acc(float (&acc)[VPL], const int32_t* __r
                                            const float* __restrict__ X, int ldx, int col,
                                            const float* __restrict__ X2 = nullptr) {
   int p = p0;
-  for (; p + U <= p1; p += U) {
+  for (; p1 - p >= U; p += U) {
     int c[U];
     float v[U];
 #pragma unroll

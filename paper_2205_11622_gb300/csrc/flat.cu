@@ -313,9 +313,9 @@ __global__ void __launch_bounds__(kFlatThreads, flat_ctas<NCH, MODE>()) k_flat(c
   int rnext = p < p1 ? a.first[w] : a.nrows;  // rows before it start before nonzero p
   int b, b1;             // pos[rnext + gl], pos[rnext + gl + 1], loaded ahead
   auto peek = [&]() {
-    const int r = rnext + gl;
-    b = r < a.nrows ? __ldg(a.pos + r) : INT_MAX;
-    b1 = r < a.nrows ? __ldg(a.pos + r + 1) : INT_MAX;
+    const unsigned r = item(rnext, gl);
+    b = r < (unsigned)a.nrows ? __ldg(a.pos + r) : INT_MAX;
+    b1 = r < (unsigned)a.nrows ? __ldg(a.pos + r + 1) : INT_MAX;
   };
   peek();
   int cur = -1;               // the row being summed
@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(kFlatThreads, flat_ctas<NCH, MODE>()) k_flat(c
     dst = typename R::Ptr(a.head, a.W, gl).row((uint32_t)w);
   }
 #pragma unroll 1
-  for (int s = 0; s < a.win; s += NS, p += NS) {
+  for (int s = 0; s < a.win; s += NS) {
     if (s0 + s >= a.nnz) break;  // warp-uniform: the first group has the earliest window
     __syncwarp();
 #pragma unroll
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(kFlatThreads, flat_ctas<NCH, MODE>()) k_flat(c
     __syncwarp();
     fetch(s + NS);
     // mark the rows that start in [p, pe): GS rows of pos per group and step
-    const int pe = p + NS < p1 ? p + NS : p1;
+    const int pe = step_end(p, NS, p1);
     bool more = p < pe;
     do {
       const bool in = more && b < pe, full = in && b1 > b && b >= p;
@@ -367,6 +367,7 @@ __global__ void __launch_bounds__(kFlatThreads, flat_ctas<NCH, MODE>()) k_flat(c
       flat_batch<GS, NCH, MODE, KIND, U>(m, st, g * NS + u0, (any >> u0 & ((1u << U) - 1u)) != 0,
                                          (unsigned)(mine >> u0), live - u0, pol, acc, c, dst, cur);
     }
+    p = pe;
   }
   if (p1 <= w * a.win) return;  // a window past the end
   const bool more = __ldg(a.pos + cur + 1) > p1;

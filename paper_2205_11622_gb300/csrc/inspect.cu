@@ -29,11 +29,11 @@ namespace {
 __global__ void k_classify(int nrows, const int32_t* __restrict__ pos, WsHeader* hdr,
                            HeavyRow* __restrict__ heavy, Chunk* __restrict__ chunks, int max_heavy,
                            int max_chunks) {
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nrows; r += gridDim.x * blockDim.x) {
-    const int p0 = pos[r], p1 = pos[r + 1];
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nrows; i += (int64_t)gridDim.x * blockDim.x) {
+    const int r = (int)i, p0 = pos[i], p1 = pos[i + 1];
     const int n = p1 - p0;
     if (n <= kLightMax) continue;
-    const int nch = (n + kChunk - 1) / kChunk;
+    const int nch = pieces(n, kChunk);
     const int h = atomicAdd(&hdr->n_heavy, 1);
     const int base = atomicAdd(&hdr->n_chunks, nch);
     if (h >= max_heavy || base + nch > max_chunks) {
@@ -43,7 +43,7 @@ __global__ void k_classify(int nrows, const int32_t* __restrict__ pos, WsHeader*
     heavy[h] = HeavyRow{r, base, nch, 0};
     for (int c = 0; c < nch; ++c) {
       const int a = p0 + c * kChunk;
-      chunks[base + c] = Chunk{r, a, min(p1, a + kChunk), base + c};
+      chunks[base + c] = Chunk{r, a, step_end(a, kChunk, p1), base + c};
     }
   }
 }
@@ -68,7 +68,7 @@ __global__ void k_csf_units(int nslices, const int32_t* __restrict__ pos2,
   for (int64_t sw = warp; sw < nslices; sw += nwarps) {
     const int s = (int)sw;
     const int n = pos3[pos2[s + 1]] - pos3[pos2[s]];
-    const int nu = n > 0 ? (n + kUnitNnz - 1) / kUnitNnz : 1;
+    const int nu = n > 0 ? pieces(n, kUnitNnz) : 1;
     int base = 0;
     if (lane == 0) base = atomicAdd(&hdr->n_units, nu);
     base = __shfl_sync(0xffffffffu, base, 0);
@@ -125,7 +125,7 @@ __global__ void k_copy_levels(const int32_t* __restrict__ pos1, const int32_t* _
 // One thread per parent: checks its position range and the order and range of
 // its children's coordinates.  Ranges are clamped so a malformed array never
 // leads to an out-of-bounds read.
-__device__ void check_level(int parent, int nparents, const int32_t* __restrict__ pos, int64_t nchild,
+__device__ void check_level(int64_t parent, int64_t nparents, const int32_t* __restrict__ pos, int64_t nchild,
                             const int32_t* __restrict__ crd, int64_t dim, int* err) {
   const int64_t a = pos[parent], b = pos[parent + 1];
   if (parent == 0 && a != 0) atomicOr(err, kErrPos);
@@ -144,25 +144,25 @@ __device__ void check_level(int parent, int nparents, const int32_t* __restrict_
 }
 
 __global__ void k_validate_csr(slnr_csr B, WsHeader* hdr) {
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < B.nrows; r += gridDim.x * blockDim.x)
+  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < B.nrows; r += (int64_t)gridDim.x * blockDim.x)
     check_level(r, B.nrows, B.pos, B.nnz, B.crd, B.ncols, &hdr->error);
   if (B.nrows == 0 && blockIdx.x == 0 && threadIdx.x == 0 && (B.pos[0] != 0 || B.nnz != 0))
     atomicOr(&hdr->error, kErrPos);
 }
 
 __global__ void k_validate_csf(slnr_csf3 B, WsHeader* hdr) {
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
+  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
   if (tid == 0) {
     if (B.pos1[0] != 0 || B.pos1[1] != B.nslices) atomicOr(&hdr->error, kErrPos);
     if (B.nslices == 0 && (B.nfibers != 0 || B.nnz != 0)) atomicOr(&hdr->error, kErrPos);
   }
-  for (int q = tid; q < B.nslices; q += nth) {
+  for (int64_t q = tid; q < B.nslices; q += nth) {
     const int64_t i = B.crd1[q];
     if (i < 0 || i >= B.dim[0]) atomicOr(&hdr->error, kErrCrdRange);
     if (q > 0 && B.crd1[q - 1] >= i) atomicOr(&hdr->error, kErrCrdOrder);
     check_level(q, B.nslices, B.pos2, B.nfibers, B.crd2, B.dim[1], &hdr->error);
   }
-  for (int f = tid; f < B.nfibers; f += nth)
+  for (int64_t f = tid; f < B.nfibers; f += nth)
     check_level(f, B.nfibers, B.pos3, B.nnz, B.crd3, B.dim[2], &hdr->error);
 }
 

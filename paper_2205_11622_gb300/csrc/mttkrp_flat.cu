@@ -163,15 +163,16 @@ __global__ void __launch_bounds__(kMtThreads, NCH == 1 ? kMtCtas : 2) k_mt(const
   bool head = slice_start(a, sl) < q;
   int send = slice_start(a, sl + 1), tail = -1;
   // a step's nonzero of this lane, and the starts and j of fibers f + 1 .. f + 32 (past the last: never)
-  int s, jn, j0, kk;
+  unsigned s;
+  int jn, j0, kk;
   float vv;
   auto fetch = [&](int p0) {
-    const int fm = f + 1 + lane, p = p0 + lane;
-    s = fm <= a.nfibers ? __ldg(a.pos3 + fm) : INT_MAX;
-    jn = fm < a.nfibers ? __ldg(a.crd2 + fm) : 0;
+    const unsigned fm = item(f, 1 + lane), p = item(p0, lane);
+    s = fm <= (unsigned)a.nfibers ? (unsigned)__ldg(a.pos3 + fm) : ~0u;
+    jn = fm < (unsigned)a.nfibers ? __ldg(a.crd2 + fm) : 0;
     j0 = f < a.nfibers ? __ldg(a.crd2 + f) : 0;
-    kk = p < pend ? flat::ld_once(a.crd3 + p, pol) : 0;
-    vv = p < pend ? flat::ld_once(a.vals + p, pol) : 0.f;
+    kk = p < (unsigned)pend ? flat::ld_once(a.crd3 + p, pol) : 0;
+    vv = p < (unsigned)pend ? flat::ld_once(a.vals + p, pol) : 0.f;
   };
   fetch(q);
   R acc;
@@ -179,25 +180,25 @@ __global__ void __launch_bounds__(kMtThreads, NCH == 1 ? kMtCtas : 2) k_mt(const
   while (q < pend) {
     const int hi = send < pend ? send : pend;
     while (q < hi) {  // warp-uniform
-      const int s31 = __shfl_sync(kFull, s, 31);
-      int qe = q + 32 < hi ? q + 32 : hi;
-      qe = s31 < qe ? s31 : qe;  // labels stay inside the 32 starts
+      const unsigned s31 = __shfl_sync(kFull, s, 31);
+      int qe = step_end(q, 32, hi);
+      qe = s31 < (unsigned)qe ? (int)s31 : qe;  // labels stay inside the 32 starts
       const int n = qe - q;
       // the nonzeros where fibers start, and each lane's count of starts at or before its own
-      const bool near = (unsigned)(s - q) < 32u;
-      unsigned at = __reduce_or_sync(kFull, near ? 1u << (s - q) : 0u);
+      const bool near = s - (unsigned)q < 32u;
+      unsigned at = __reduce_or_sync(kFull, near ? 1u << (s - (unsigned)q) : 0u);
       int cnt = __popc(at & (2u << lane) - 1u);
       if (__popc(__ballot_sync(kFull, near)) != __popc(at)) {  // empty fibers share a start: count them all
         cnt = 0;
 #pragma unroll
         for (int step = 16; step > 0; step >>= 1)
-          if (__shfl_sync(kFull, s, cnt + step - 1) <= q + lane) cnt += step;
+          if (__shfl_sync(kFull, s, cnt + step - 1) <= item(q, lane)) cnt += step;
       }
       const int jx = __shfl_sync(kFull, jn, cnt > 0 ? cnt - 1 : 0);
       __syncwarp();
       kv[wib][lane] = make_int2(kk, __float_as_int(vv));
       js[wib][lane] = cnt > 0 ? jx : j0;
-      f += __popc(__ballot_sync(kFull, s <= qe));  // the fiber holding qe
+      f += __popc(__ballot_sync(kFull, s <= (unsigned)qe));  // the fiber holding qe
       __syncwarp();
       fetch(qe);  // the next step's, in flight with this one's rows
       at |= kBlocks;  // every group begins a run at its first nonzero ...

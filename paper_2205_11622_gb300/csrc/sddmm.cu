@@ -48,8 +48,8 @@ __device__ __forceinline__ void sddmm_spmm_range(float (&acc)[RowLanes<WM>::VPL]
     bool ok[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int p = p0 + base + u * RL::GPW + grp;
-      ok[u] = p < p1;
+      const unsigned p = item(p0, base + u * RL::GPW + grp);
+      ok[u] = p < (unsigned)p1;
       cc[u] = ok[u] ? __ldg(crd + p) : 0;
       vv[u] = ok[u] ? __ldg(vals + p) : 0.f;
     }
@@ -92,15 +92,15 @@ __device__ __forceinline__ void short_row_range(float (&acc)[RowLanes<WM>::VPL],
   using RL = RowLanes<WM>;
   constexpr int VPL = RL::VPL;
   for (int it = 0; it < maxlen; it += U) {
-    const int base = p0 + it;
     int cc[U];
     float vv[U];
     bool ok[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      ok[u] = base + u < p1;
-      cc[u] = ok[u] ? __ldg(crd + base + u) : 0;
-      vv[u] = ok[u] ? __ldg(vals + base + u) : 0.f;
+      const unsigned p = item(p0, it + u);
+      ok[u] = p < (unsigned)p1;
+      cc[u] = ok[u] ? __ldg(crd + p) : 0;
+      vv[u] = ok[u] ? __ldg(vals + p) : 0.f;
     }
     float d[U][VPL], e[U][VPL];
 #pragma unroll
@@ -266,8 +266,8 @@ __device__ __forceinline__ void sddmm_range(const float (&c)[RowLanes<W>::VPL], 
   using RL = RowLanes<W>;
   const int n = p1 - p0;
   for (int base = 0; base < n; base += RL::GPW) {
-    const int p = p0 + base + grp;
-    const bool ok = p < p1;
+    const unsigned p = item(p0, base + grp);
+    const bool ok = p < (unsigned)p1;
     float d[RL::VPL];
     if (ok) ldg_vec<RL::VPL>(d, D + (int64_t)__ldg(crd + p) * W + col); else zero_vec(d);
     float dot = 0.f;

@@ -38,7 +38,7 @@ constexpr int kScanRows = 2048;
 constexpr int kScanThreads = 256;
 constexpr int kRowsPerThread = kScanRows / kScanThreads;
 
-__device__ __forceinline__ int segs_of(int n) { return n <= kSegChunk ? 1 : (n + kSegChunk - 1) / kSegChunk; }
+__device__ __forceinline__ int segs_of(int n) { return n <= kSegChunk ? 1 : pieces(n, kSegChunk); }
 
 // Segments are listed by length class, longest first, so that the items a
 // lane group takes together have similar lengths and one batch shape fits
@@ -430,10 +430,11 @@ __device__ __forceinline__ bool short_wave(unsigned gmask, int gbase, int gl, in
   for (int h = 0; h < SPL; ++h) {
     const int t = gl + h * GS, w = t / N < W ? t / N : W - 1, s = t % N;
     const int p0 = __shfl_sync(gmask, rp0, gbase + w0 + w), p1 = __shfl_sync(gmask, rp1, gbase + w0 + w);
-    const bool ok = t < S && p0 + s < p1;
+    const unsigned p = item(p0, s);
+    const bool ok = t < S && p < (unsigned)p1;
     const uint64_t pol = stream_policy();
-    mc[h] = ok ? ld_stream(crd + p0 + s, pol) : -1;
-    mv[h] = ok ? ld_stream(vals + p0 + s, pol) : 0.f;
+    mc[h] = ok ? ld_stream(crd + p, pol) : -1;
+    mv[h] = ok ? ld_stream(vals + p, pol) : 0.f;
   }
   float x[S][VPL];
 #pragma unroll
@@ -483,7 +484,7 @@ __device__ __forceinline__ bool long_items(unsigned gmask, int gbase, int gl, in
   auto p1_of = [&](int r) { return __shfl_sync(gmask, rp1, gbase + r); };
   // a chunk is item r's nonzeros [q, min(q + GS, p1(r))); r == R: none left
   auto advance = [&](int& r, int& q) {
-    if (r < R && q + GS < p1_of(r)) {
+    if (r < R && inside(q, GS, p1_of(r))) {
       q += GS;
     } else {
       ++r;
@@ -491,10 +492,11 @@ __device__ __forceinline__ bool long_items(unsigned gmask, int gbase, int gl, in
     }
   };
   auto load_idx = [&](int r, int q, int& ic, float& iv) {
-    const bool ok = r < R && q + gl < p1_of(r);
+    const unsigned p = item(q, gl);
+    const bool ok = r < R && p < (unsigned)p1_of(r);
     const uint64_t pol = stream_policy();
-    ic = ok ? ld_stream(crd + q + gl, pol) : -1;
-    iv = ok ? ld_stream(vals + q + gl, pol) : 0.f;
+    ic = ok ? ld_stream(crd + p, pol) : -1;
+    iv = ok ? ld_stream(vals + p, pol) : 0.f;
   };
   int r = 0, q = p0_of(0);  // current chunk
   int rn = r, qn = q;       // next chunk

@@ -63,7 +63,7 @@ __device__ __forceinline__ void wgather(float4 (&acc)[NCH], const int32_t* __res
                                         const float* __restrict__ X2, int W, int lane) {
   wzero(acc);
   int p = p0;
-  for (; p + 2 <= p1; p += 2) {
+  for (; p1 - p >= 2; p += 2) {
     const int c0 = __ldg(crd + p), c1 = __ldg(crd + p + 1);
     const float v0 = __ldg(vals + p), v1 = __ldg(vals + p + 1);
     float4 x0[NCH], x1[NCH];
@@ -297,8 +297,8 @@ __device__ __forceinline__ void w_sddmm_row(float4 (&acc)[NCH], const float* cs,
   for (int i = 0; i < NCH; ++i)
     c[i] = 4 * (lane + 32 * i) < Kd ? reinterpret_cast<const float4*>(cs)[lane + 32 * i]
                                      : make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int p = p0; p < p1; p += 2) {
-    const bool two = p + 1 < p1;
+  for (unsigned p = (unsigned)p0; p < (unsigned)p1; p += 2) {
+    const bool two = p + 1 < (unsigned)p1;
     const int j0 = __ldg(crd + p), j1 = two ? __ldg(crd + p + 1) : j0;
     float4 d0[NCH], d1[NCH];
     wload(d0, D + (int64_t)j0 * Kd, Kd, lane);
