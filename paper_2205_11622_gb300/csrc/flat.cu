@@ -134,23 +134,7 @@ __global__ void __launch_bounds__(kRowsThreads) k_flat_rows(const FlatArgs a) {
     const int b = __ffs(m) - 1, lo = __shfl_sync(FULL, w0, b), hi = __shfl_sync(FULL, w1, b);
     for (int w = lo + lane; w < hi; w += 32) a.first[w] = (int)r0 + b;
   }
-  const int w4 = a.W >> 2;
-  float4* base = reinterpret_cast<float4*>(a.out + r0 * a.W);
-  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-  const unsigned m = __ballot_sync(FULL, in && p0 == p1);
-  if (m == FULL) {
-    for (int i = lane; i < 32 * w4; i += 32) base[i] = z;
-    return;
-  }
-  if (__popc(m) * ceil_div(w4, 32) > w4) {  // narrow rows: 32 / w4 of them a step
-    for (int i = lane; i < 32 * w4; i += 32)
-      if (m >> (i / w4) & 1u) base[i] = z;
-    return;
-  }
-  for (unsigned k = m; k != 0; k &= k - 1) {
-    const int b = __ffs(k) - 1;
-    for (int i = lane; i < w4; i += 32) base[b * w4 + i] = z;
-  }
+  flat::zero_rows(a.out + r0 * a.W, a.W, __ballot_sync(FULL, in && p0 == p1), lane);
 }
 
 // One warp's staged nonzeros: entry i belongs to window i / NS of the warp.

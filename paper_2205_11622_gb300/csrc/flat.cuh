@@ -66,6 +66,27 @@ __device__ __forceinline__ float ld_once(const float* p, uint64_t pol) {
   return v;
 }
 
+// Zeroes the rows of `rows` (of 32, W values each, from base on) whose bit of m
+// is set; by a whole warp.
+__device__ __forceinline__ void zero_rows(float* rows, int W, unsigned m, int lane) {
+  const int w4 = W >> 2;
+  float4* base = reinterpret_cast<float4*>(rows);
+  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (m == 0xffffffffu) {
+    for (int i = lane; i < 32 * w4; i += 32) base[i] = z;
+    return;
+  }
+  if (__popc(m) * ceil_div(w4, 32) > w4) {  // narrow rows: 32 / w4 of them a step
+    for (int i = lane; i < 32 * w4; i += 32)
+      if (m >> (i / w4) & 1u) base[i] = z;
+    return;
+  }
+  for (; m != 0; m &= m - 1) {
+    const int b = __ffs(m) - 1;
+    for (int i = lane; i < w4; i += 32) base[b * w4 + i] = z;
+  }
+}
+
 // How the columns of a row are spread over its lane group.
 enum RowKind {
   kWhole = 0,  // W = 8 GS NCH: every lane holds columns; 32-byte accesses

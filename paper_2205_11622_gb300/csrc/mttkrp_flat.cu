@@ -115,11 +115,7 @@ __global__ void __launch_bounds__(kFirstThreads) k_mt_first(const MtArgs a, int 
               s = __shfl_sync(kFull, q, b);
     for (int w = lo + lane; w < hi; w += 32) a.first_slice[w] = s;
   }
-  const int w4 = a.M >> 2;
-  for (unsigned m = __ballot_sync(kFull, in && p0 == p1); m != 0; m &= m - 1) {
-    float4* row = reinterpret_cast<float4*>(a.A + (i0 + __ffs(m) - 1) * a.M);
-    for (int c = lane; c < w4; c += 32) row[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-  }
+  flat::zero_rows(a.A + i0 * a.M, a.M, __ballot_sync(kFull, in && p0 == p1), lane);
 }
 
 // Slice s's row is finished (every group of the warp holds it): row crd1[s] of
