@@ -362,17 +362,24 @@ __global__ void __launch_bounds__(kFlatThreads, flat_ctas<NCH, MODE>()) k_flat(c
 
 // Rows that span windows: out(r,:) = tail of the window where r starts + the
 // heads of the windows after it up to r's last nonzero, in that order.  A CTA
-// looks at 256 windows; rows of more than kLongRow heads are summed by the
-// whole CTA (lane groups take heads g, g + G, ... in order, then a fixed
-// pairwise tree), the others by a lane group each.
+// looks at four windows a lane group (at most one a thread), so that wide rows
+// are not one group's chain (<SDDMM,SpMM> 30k rows 100/48: 78 us with 256
+// windows, 72 with 64; 3k 64/64 24.3 | 22.6); rows of more than kLongRow heads
+// are summed by the whole CTA (lane groups take heads g, g + G, ... in order,
+// then a fixed pairwise tree), the others by a lane group each.
 constexpr int kCombineThreads = 256;
+template <int GS>
+constexpr int combine_windows() {
+  return 4 * (kCombineThreads / GS) < kCombineThreads ? 4 * (kCombineThreads / GS) : kCombineThreads;
+}
 constexpr int kLongRow = 32;
 
 template <int GS, int NCH, int KIND>
 __global__ void __launch_bounds__(kCombineThreads) k_flat_combine(FlatArgs a) {
   using R = Row<GS, NCH, KIND>;
   constexpr int G = kCombineThreads / GS;  // lane groups of the CTA
-  __shared__ int2 item[kCombineThreads];   // {window, heads}: short rows from the front, long ones from the back
+  constexpr int N = combine_windows<GS>();
+  __shared__ int2 item[N];  // {window, heads}: short rows from the front, long ones from the back
   __shared__ int nshort, nlong;
   __shared__ u64 red[kCombineThreads * R::P];
   const int tid = threadIdx.x, g = tid / GS, gl = tid % GS;
@@ -381,18 +388,18 @@ __global__ void __launch_bounds__(kCombineThreads) k_flat_combine(FlatArgs a) {
   flat::grid_wait();  // k_flat's pieces
   __syncthreads();
   {
-    const int64_t w = (int64_t)blockIdx.x * kCombineThreads + tid;
-    const int r = w < a.nw ? a.tail_row[w] : -1;
+    const int64_t w = (int64_t)blockIdx.x * N + tid;
+    const int r = tid < N && w < a.nw ? a.tail_row[w] : -1;
     if (r >= 0) {
       const int n = (int)((__ldg(a.pos + r + 1) - 1) / a.win - w);
-      const int at = n > kLongRow ? kCombineThreads - 1 - atomicAdd(&nlong, 1) : atomicAdd(&nshort, 1);
+      const int at = n > kLongRow ? N - 1 - atomicAdd(&nlong, 1) : atomicAdd(&nshort, 1);
       item[at] = make_int2((int)w, n);
     }
   }
   __syncthreads();
   const int ns = nshort, nl = nlong;
   for (int i = 0; i < nl; ++i) {
-    const int2 it = item[kCombineThreads - 1 - i];
+    const int2 it = item[N - 1 - i];
     const uint32_t h = (uint32_t)it.x + 1;  // the first head
     R acc;
     acc.zero();
@@ -459,7 +466,7 @@ cudaError_t flat_launch(const FlatArgs& a, cudaStream_t s) {
       flat::launch_early(k_flat<GS, NCH, MODE, KIND>,
                          SLNR_COUNTED(ceil_div(ceil_div(a.nw, 32 / GS), kFlatThreads / 32)), kFlatThreads, 0, s, a);
   if (e != cudaSuccess || a.nw < 2) return e;
-  return flat::launch_early(k_flat_combine<GS, NCH, KIND>, SLNR_COUNTED(ceil_div(a.nw, kCombineThreads)),
+  return flat::launch_early(k_flat_combine<GS, NCH, KIND>, SLNR_COUNTED(ceil_div(a.nw, combine_windows<GS>())),
                             kCombineThreads, 0, s, a);
 }
 

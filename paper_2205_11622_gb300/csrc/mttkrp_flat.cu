@@ -275,15 +275,21 @@ __global__ void __launch_bounds__(kMtThreads, NCH == 1 ? kMtCtas : 2) k_mt(const
   if (lane == 0) a.tail_slice[w] = tail;
 }
 
-// Slices that span windows: tail + heads in window order.  A CTA looks at as
-// many windows as it has threads; slices of more than kMtLong heads are summed
-// by the whole CTA (lane groups take heads g, g + G, ... in order, then their
-// sums are added in order), the others by a warp each (its groups the same
-// way).  CTAs are large, so that the hub slice (3900 heads of 10M nonzeros) is
-// a few rounds of loads long.
+// Slices that span windows: tail + heads in window order.  A CTA looks at four
+// windows a warp; slices of more than kMtLong heads are summed by the whole CTA
+// (lane groups take heads g, g + G, ... in order, then their sums are added in
+// order), the others by a warp each (its groups the same way).  CTAs are large,
+// so that the hub slice (3900 heads of 10M nonzeros) is a few rounds of loads
+// long, and look at few windows, so that short slices are not one warp's chain
+// (20k slices of 200 nonzeros, rank 16: 100 us with a window a thread, 72 with
+// four a warp; 10k slices of 1000, rank 32: 157 | 151).
 template <int NCH>
 constexpr int mt_combine_threads() {
   return NCH == 1 ? 1024 : 256;  // 32 KB of shared memory
+}
+template <int NCH>
+constexpr int mt_combine_windows() {
+  return mt_combine_threads<NCH>() / 8;
 }
 constexpr int kMtLong = 64;
 
@@ -291,8 +297,8 @@ template <int GS, int NCH, int KIND>
 __global__ void __launch_bounds__(mt_combine_threads<NCH>()) k_mt_combine(const MtArgs a) {
   using R = Row<GS, NCH, KIND>;
   constexpr int kMtCombineThreads = mt_combine_threads<NCH>();
-  constexpr int W = kMtCombineThreads / 32, GW = 32 / GS;
-  __shared__ int2 item[kMtCombineThreads];
+  constexpr int W = kMtCombineThreads / 32, GW = 32 / GS, N = mt_combine_windows<NCH>();
+  __shared__ int2 item[N];
   __shared__ int nshort, nlong;
   __shared__ u64 red[W][32 * R::P];
   const int tid = threadIdx.x, wib = tid >> 5, lane = tid & 31, g = lane / GS, gl = lane % GS;
@@ -301,11 +307,11 @@ __global__ void __launch_bounds__(mt_combine_threads<NCH>()) k_mt_combine(const 
   flat::grid_wait();  // k_mt's pieces
   __syncthreads();
   {
-    const int64_t w = (int64_t)blockIdx.x * kMtCombineThreads + tid;
-    const int s = w < a.nw ? a.tail_slice[w] : -1;
+    const int64_t w = (int64_t)blockIdx.x * N + tid;
+    const int s = tid < N && w < a.nw ? a.tail_slice[w] : -1;
     if (s >= 0) {
       const int n = ((slice_start(a, s + 1) - 1) >> a.shift) - (int)w;
-      const int at = n > kMtLong ? kMtCombineThreads - 1 - atomicAdd(&nlong, 1) : atomicAdd(&nshort, 1);
+      const int at = n > kMtLong ? N - 1 - atomicAdd(&nlong, 1) : atomicAdd(&nshort, 1);
       item[at] = make_int2((int)w, n);
     }
   }
@@ -328,7 +334,7 @@ __global__ void __launch_bounds__(mt_combine_threads<NCH>()) k_mt_combine(const 
     }
   };
   for (int i = 0; i < nl; ++i) {
-    const int2 it = item[kMtCombineThreads - 1 - i];
+    const int2 it = item[N - 1 - i];
     R acc;
     acc.zero();
     if (wib == 0 && g == 0) acc.load_written(tails, (uint32_t)it.x);
@@ -367,8 +373,8 @@ cudaError_t mt_launch(const MtArgs& a, cudaStream_t s) {
   cudaError_t e =
       flat::launch_early(k_mt<GS, NCH, KIND>, SLNR_COUNTED(ceil_div(a.nw, kMtWarps)), kMtThreads, 0, s, a);
   if (e != cudaSuccess || a.nw < 2) return e;
-  constexpr int threads = mt_combine_threads<NCH>();
-  return flat::launch_early(k_mt_combine<GS, NCH, KIND>, SLNR_COUNTED(ceil_div(a.nw, threads)), threads, 0, s, a);
+  return flat::launch_early(k_mt_combine<GS, NCH, KIND>, SLNR_COUNTED(ceil_div(a.nw, mt_combine_windows<NCH>())),
+                            mt_combine_threads<NCH>(), 0, s, a);
 }
 
 template <int KIND>
