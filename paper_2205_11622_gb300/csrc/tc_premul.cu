@@ -58,10 +58,29 @@ __device__ __forceinline__ bool pt_wait(uint64_t* bar, uint32_t parity, long lon
   return true;
 }
 
-__device__ __forceinline__ void pt_split(float x, uint32_t& hi, uint32_t& lo) {
-  hi = tc::to_tf32(x);
-  const bool finite = (hi & 0x7F800000u) != 0x7F800000u;
-  lo = finite ? tc::to_tf32(x - __uint_as_float(hi)) : 0u;
+// v as the sum of two tf32 values each.  Infinities and NaN have no second
+// part; the largest finite values, which would round to infinity, are cut off.
+__device__ __forceinline__ void pt_split(const float4& v, uint4& hi, uint4& lo) {
+  const float x[4] = {v.x, v.y, v.z, v.w};
+  uint32_t h[4], l[4], most = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    h[i] = tc::to_tf32(x[i]);
+    l[i] = tc::to_tf32(x[i] - __uint_as_float(h[i]));
+    most = max(most, h[i] & 0x7FFFFFFFu);
+  }
+  if (most >= 0x7F800000u) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if ((h[i] & 0x7F800000u) != 0x7F800000u) continue;
+      const uint32_t bits = __float_as_uint(x[i]);
+      const bool finite = (bits & 0x7F800000u) != 0x7F800000u;
+      if (finite) h[i] = bits & 0xFFFFE000u;
+      l[i] = finite ? tc::to_tf32(x[i] - __uint_as_float(h[i])) : 0u;
+    }
+  }
+  hi = make_uint4(h[0], h[1], h[2], h[3]);
+  lo = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
 template <int K, int L, bool H>
@@ -157,10 +176,7 @@ __global__ void __launch_bounds__(kPtThreads, 1)
           float4 v = x[u][i];
           if constexpr (H) v = make_float4(v.x * y[u][i].x, v.y * y[u][i].y, v.z * y[u][i].z, v.w * y[u][i].w);
           uint4 hi, lo;
-          pt_split(v.x, hi.x, lo.x);
-          pt_split(v.y, hi.y, lo.y);
-          pt_split(v.z, hi.z, lo.z);
-          pt_split(v.w, hi.w, lo.w);
+          pt_split(v, hi, lo);
           const int r = 8 * warp + 4 * i + lr, off = r * 128 + ((lc ^ (r & 7)) << 4);
           *reinterpret_cast<uint4*>(s + off) = hi;
           *reinterpret_cast<uint4*>(s + kPtBlock + off) = lo;

@@ -218,6 +218,28 @@ def test_split_product_infinities(slnr, where):
     assert np.array_equal(np.isposinf(out), hit) and np.isfinite(out[~hit]).all()
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("two", [False, True])
+def test_split_product_largest_values(slnr, two):
+    # the largest finite values of X (masks), whose upper part must not round to infinity: D of 2^-12 and zeros keeps
+    # every sum finite, and 0 times them is 0
+    w = columns_workload(500, 64, 64, two)
+    most = np.finfo(np.float32).max
+    w.dense["C"][3] = np.where(np.arange(64) % 2, most, -most)
+    w.dense["C"][4, 5] = most
+    if two:
+        w.dense["D"][3:5] = 1
+    D = w.dense["E" if two else "D"]
+    D[:] = 2.0 ** -12
+    D[:, ::3] = 0
+    w.B.vals[:] *= 0.5
+    ref, ref_abs = oracle.get().run(w)
+    dB, dd = P.to_device(w)
+    out = slnr.run(w.op, dB, dd, allow_tf32=True).cpu().numpy()
+    assert np.isfinite(ref).all() and not out[:, ::3].any()
+    assert P.rel_err(out, ref, ref_abs) <= 1e-5
+
+
 def csf(kind, rng, d1, d2, seed):
     """CSF tensors whose slices and fibers end at window edges, span many windows, or are empty in runs."""
     if kind == "few":            # fewer nonzeros than a window
