@@ -59,6 +59,55 @@ def values_of(op, out):
     return out[4] if op == "spttm_ttm" else out
 
 
+# The expressions that multiply by a dense matrix last, or by it first (X . D once per gathered row, then the sums):
+# the operands whose rows are gathered.
+GATHERED = {"spmm_gemm": ("C",), "spttm_ttm": ("C",), "spmmh_gemm": ("C", "D"), "sddmm_spmm_gemm": ("D", "F")}
+
+
+def row_first(w):
+    """w with more columns (a longer third mode) than nonzeros: the same result, by the kernels that go row by row.
+
+    No nonzero is in the new columns; their rows of the gathered operands are NaN."""
+    import workloads as wl
+    B, op = w.B, w.op
+    ncols = B.dims[2] if op == "spttm_ttm" else B.ncols
+    extra = B.nnz + 1 - ncols
+    if extra <= 0:
+        return w
+    dense = dict(w.dense)
+    for name in GATHERED[op]:
+        x = dense[name]
+        dense[name] = np.concatenate([x, np.full((extra, x.shape[1]), np.nan, np.float32)])
+    if op == "spttm_ttm":
+        B = wl.CSF3((*B.dims[:2], ncols + extra), B.pos1, B.crd1, B.pos2, B.crd2, B.pos3, B.crd3, B.vals)
+    else:
+        B = wl.CSR(B.nrows, ncols + extra, B.pos, B.crd, B.vals)
+    return wl.Workload(w.name + "_row_first", op, B, dense, w.dims)
+
+
+def phases(w, **kw):
+    """(output values, names of the phases) of one call; no device flag may be set."""
+    import paper_2205_11622_gb300 as slnr
+    B, dense = to_device(w)
+    slnr.timing_enable(True)
+    try:
+        out = slnr.run(w.op, B, dense, **kw)
+        names = [n for n, _ in slnr.timing_read()]
+    finally:
+        slnr.timing_enable(False)
+    assert slnr.device_flags() == 0, f"device flags {slnr.device_flags():#x}"
+    return values_of(w.op, out), names
+
+
+def check_row_first(w, allow_tf32, ref, ref_abs, tol):
+    """The fused call of w's expression on the row-by-row kernels, against w's reference."""
+    got, names = phases(row_first(w), allow_tf32=allow_tf32)
+    assert not any("premul" in n or n.startswith("flat_") for n in names), names
+    err = rel_err(got.cpu().numpy(), ref, ref_abs)
+    assert err <= tol, f"{w.name} row first tf32={allow_tf32}: err {err:.3e} > {tol:.1e}"
+    return names
+
+
 def uses_tensor_cores(op, variant="fused") -> bool:
     """Whether the call may contract on TF32 tensor cores when allowed: the
     fused and unfused <SpMM,GEMM>, <SpTTM,SpTTM>, <SpMMH,GEMM> and

@@ -29,18 +29,6 @@ def gpu():
     slnr.lib()
 
 
-def phases(w, B, dense, **kw):
-    """(output values, names of the call's phases)."""
-    slnr.timing_enable(True)
-    try:
-        out = slnr.run(w.op, B, dense, **kw)
-        names = [n for n, _ in slnr.timing_read()]
-    finally:
-        slnr.timing_enable(False)
-    assert slnr.device_flags() == 0
-    return P.values_of(w.op, out), names
-
-
 def csr_of(lens, ncols, seed):
     """Rows of the given lengths: distinct columns a + b t mod ncols, sorted."""
     rng = np.random.default_rng(seed)
@@ -116,8 +104,7 @@ def test_tf32_values_stay_where_rows_are_long(gpu, op, K, L):
     lens = np.full(n, 1)
     lens[5] = 50000
     w = workload(op, lens.tolist(), ncols, K, L, 0x51A4 + K)
-    B, dense = P.to_device(w)
-    got, _ = phases(w, B, dense, allow_tf32=True)
+    got, _ = P.phases(w, allow_tf32=True)
     ref = row_first(w)
     rms = np.sqrt(np.mean(ref ** 2))
     assert np.max(np.abs(got.cpu().numpy() - ref) / np.maximum(rms, np.abs(ref))) <= 5e-3
@@ -154,13 +141,13 @@ def test_hadamard_product_first_gives_the_same_bits(gpu, n, K, L):
     lens[7] = 40000
     w = workload("spmmh_gemm", lens.tolist(), n, K, L, 0x51A4 + n)
     B, d = P.to_device(w)
-    got, names = phases(w, B, d, allow_tf32=True)
+    got, names = P.phases(w, allow_tf32=True)
     assert names == ["seg_count", "seg_write", "hadamard", "tc_spmm_gemm", "combine"]
     assert torch.equal(got, slnr.spmm_gemm(B, d["C"] * d["D"], d["E"], allow_tf32=True))
     # three nonzeros a column: the products in the kernel's gathers
     few = workload("spmmh_gemm", [3] * n, n, 64, L, 0x51A4 + n)
     B, d = P.to_device(few)
-    got, names = phases(few, B, d, allow_tf32=True)
+    got, names = P.phases(few, allow_tf32=True)
     if n > 1 << 17:
         assert "tc_spmmh_gemm" in names
         assert torch.equal(got, slnr.spmm_gemm(B, d["C"] * d["D"], d["E"], allow_tf32=True))
@@ -176,8 +163,7 @@ def test_sampled_gemm_stays_fp32_at_widths_without_a_tensor_core_kernel(gpu, K, 
     w = wl.Workload("sampled", "sddmm_spmm_gemm", B, {"C": wl.normal(r, (n, K)), "D": wl.normal(r, (n, K)),
                                                       "F": wl.normal(r, (n, L)), "W": wl.normal(r, (L, M))},
                     {"K": K, "L": L, "M": M})
-    dB, d = P.to_device(w)
-    assert torch.equal(phases(w, dB, d, allow_tf32=True)[0], phases(w, dB, d, allow_tf32=False)[0])
+    assert torch.equal(P.phases(w, allow_tf32=True)[0], P.phases(w, allow_tf32=False)[0])
 
 
 @pytest.mark.parametrize("op,nrows,ncols,nnz,sizes,tf32,first", [
@@ -221,10 +207,10 @@ def test_a_workspace_that_holds_row_first_is_enough(gpu, op, K, L, row_kernel):
     ref, ref_abs = oracle.get().run(w)
     own = slnr.Workspace()
     small = workload(op, [5] * 100, n if op != "spttm_ttm" else 1000, K, L, 1)
-    phases(small, *P.to_device(small), workspace=own)
-    full, names = phases(w, B, d, workspace=own)  # a small call's workspace before it: the order is the same
+    P.phases(small, workspace=own)
+    full, names = P.phases(w, workspace=own)  # a small call's workspace before it: the order is the same
     assert names[-1].startswith("flat_"), names
-    rows, names = phases(w, B, d, workspace=Scarce(own.buf.numel() // 2))
+    rows, names = P.phases(w, workspace=Scarce(own.buf.numel() // 2))
     assert row_kernel in names, names
     for got in (full, rows):
         assert P.rel_err(got.cpu().numpy(), ref, ref_abs) <= P.TOL_TF32
@@ -236,3 +222,56 @@ def test_a_workspace_that_holds_row_first_is_enough(gpu, op, K, L, row_kernel):
     with pytest.raises(slnr.SlnrError) as e:
         slnr.run(op, B, d, workspace=ws)
     assert e.value.status == 4
+
+
+# Rows at the row kernels' edges: 127/128/129 straddle the tensor-core segment length, 255/256/257 the light/heavy
+# boundary, 5000 is a long heavy row; runs of short rows fill waves and tiles, the number of rows is ragged.
+EDGES = ([127, 128, 129, 255, 256, 257, 5000, 1, 0, 3] + [1, 2, 3, 4, 5, 7, 8, 9, 16, 17] * 130 + [0] * 60 + [64, 65, 33] * 11)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("op,K,L", [
+    *(("spmm_gemm", *w) for w in [(16, 16), (16, 256), (32, 32), (32, 128), (64, 16), (64, 64), (128, 64), (128, 128),
+                                  (128, 256), (256, 16), (256, 64)]),
+    *(("spmmh_gemm", *w) for w in [(16, 64), (32, 16), (64, 64), (128, 128), (128, 256), (256, 32)]),
+    *(("sddmm_spmm_gemm", *w) for w in [(32, 32), (32, 128), (64, 64), (128, 32), (128, 128)]),
+    *(("spttm_ttm", *w) for w in [(16, 16), (64, 64), (128, 128), (256, 64)])])
+def test_tensor_core_row_kernel_edges(gpu, op, K, L):
+    w = workload(op, EDGES, 6000, K, L, 0x51A4 + K + L)
+    assert w.B.nnz >= 1 << 14
+    ref, ref_abs = oracle.get().run(w)
+    names = P.check_row_first(w, True, ref, ref_abs, P.TOL_TF32)
+    assert ("tc_spmm_gemm" if op == "spttm_ttm" else f"tc_{op}") in names, names
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("op,K,L,kernel", [
+    ("spmm_gemm", 64, 64, "spmm_gemm_tiles"), ("spmm_gemm", 4, 8, "spmm_gemm_tiles"), ("spmm_gemm", 128, 256, "spmm_gemm_tiles"),
+    ("spmm_gemm", 100, 36, "w_spmm_gemm_tiles"), ("spmm_gemm", 512, 64, "w_spmm_gemm_tiles"),
+    ("spmmh_gemm", 64, 64, "spmm_gemm_tiles"), ("spmmh_gemm", 36, 100, "w_spmm_gemm_tiles"),
+    ("sddmm_spmm_gemm", 64, 64, "sddmm_spmm_gemm_tiles"), ("sddmm_spmm_gemm", 8, 32, "sddmm_spmm_gemm_tiles"),
+    ("sddmm_spmm_gemm", 256, 16, "sddmm_spmm_gemm_tiles"), ("sddmm_spmm_gemm", 100, 36, "w_sddmm_spmm_gemm_tiles"),
+    ("spttm_ttm", 64, 32, "spmm_gemm_tiles"), ("spttm_ttm", 20, 48, "w_spmm_gemm_tiles")])
+def test_fp32_row_kernel_edges(gpu, op, K, L, kernel):
+    w = workload(op, EDGES, 6000, K, L, 0x51A4 + K + L)
+    ref, ref_abs = oracle.get().run(w)
+    names = P.check_row_first(w, False, ref, ref_abs, P.TOL_FP32)
+    assert kernel in names, names
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("L,K", [(4, 4), (4, 64), (32, 4), (8, 32), (16, 16), (64, 16), (16, 64), (64, 64)])
+def test_sddmm_spmm_row_kernel(gpu, L, K):
+    # fewer than four nonzeros a row: claims of short rows, of long ones and mixed, chunks of heavy rows
+    lens = [5000, 257, 256, 255, 9, 8, 7, 0] + [1, 0, 2, 8, 0, 3, 9, 1] * 600 + [0] * 1001
+    rng = np.random.default_rng(L + K)
+    lens = np.concatenate([lens[:8], rng.permutation(lens[8:])]).tolist()
+    r = wl.Rng(0x51A4 + L + K)
+    B = csr_of(lens, 6000, 0x51A4 + L)
+    assert B.nnz < 4 * B.nrows
+    w = wl.Workload("rows", "sddmm_spmm", B, {"C": wl.uniform(r, (B.nrows, L), -1, 1), "D": wl.uniform(r, (6000, L), -1, 1),
+                                              "E": wl.uniform(r, (6000, K), -1, 1)}, {"K": K, "L": L})
+    ref, ref_abs = oracle.get().run(w)
+    got, names = P.phases(w)
+    assert names == ["classify", "sddmm_spmm_rows", "combine"]
+    assert P.rel_err(got.cpu().numpy(), ref, ref_abs) <= P.TOL_FP32

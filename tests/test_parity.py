@@ -2,8 +2,8 @@
 
 Sizes span several row tiles, heavy rows split into chunks, ragged tails,
 empty rows / slices, every supported inner width, both variants (fused and
-unfused) and both contraction precisions (fp32 and TF32).  Everything goes
-through the C ABI (paper_2205_11622_gb300 is a ctypes binding of libslnr).
+unfused), both contraction precisions (fp32 and TF32) and, where a call may
+take its dense product first, both orders.  Everything goes through the C ABI (paper_2205_11622_gb300 is a ctypes binding of libslnr).
 """
 import numpy as np
 import pytest
@@ -46,6 +46,8 @@ def check(slnr, orc, w, variant="fused", allow_tf32=False, tol=None):
         p1, c1, p2, c2 = orc.spttm_ttm_pattern(w.B.crd1, w.B.pos2, w.B.crd2)
         for got_i, want in zip(out[:4], (p1, c1, p2, c2)):
             assert np.array_equal(got_i.cpu().numpy(), want), "output index arrays must be bit-exact"
+    if variant == "fused" and w.op in P.GATHERED:
+        P.check_row_first(w, allow_tf32, ref, ref_abs, tol)
     return out, err
 
 
@@ -82,9 +84,11 @@ def test_mttkrp_widths(slnr, orc, L, variant):
 @pytest.mark.parametrize("L", [4, 32, 256])
 @pytest.mark.parametrize("variant", ["fused", "unfused"])
 def test_mttkrp_hub_slice(slnr, orc, L, variant):
-    # Zipf(1.8) over 40 slices: 3 slices of more than 16 units (512 nonzeros
-    # each; the largest has 162, i.e. 3 runs of at most 64 units, the last one
-    # ragged) are summed in two levels, the other 37 by a warp each
+    # Zipf(1.8) over 40 slices.  Unfused: 3 slices of more than 16 units (512
+    # nonzeros each; the largest has 162, i.e. 3 runs of at most 64 units, the
+    # last one ragged) are summed in two levels, the other 37 by a warp each.
+    # Fused: the largest spans some 650 windows (summed by a whole CTA, as are
+    # those of more than 64), the others a few (a warp each) or one
     w = wl.mttkrp_zipf(0x51A5, (40, 400, 500), 150000, 1.8, L)
     check(slnr, orc, w, variant)
 
@@ -271,33 +275,38 @@ def test_single_buffer_tensor_core_path(slnr, orc, K, L, op):
     # tile into the next, over more than 150 tiles; every wait must end
     # (the device flag stays 0) and the result match the oracle
     if op == "spmm_gemm":
-        w = wl.spmm_gemm_rmat(0x51A4 + 19 * K + L, 20000, 12, K, L)
+        w = wl.spmm_gemm_rmat(0x51A4 + 19 * K + L, 20000, 4, K, L)
     else:
         w = wl.spttm_ttm_powerlaw(0x51A4 + 23 * K + L, (200, 200, 900), 100000, 8.0, 900, K, L)
-    check(slnr, orc, w, "fused", True)
+    ref, ref_abs = orc.run(w)
+    names = P.check_row_first(w, True, ref, ref_abs, P.TOL_TF32)
+    assert "tc_spmm_gemm" in names, names
 
 
 @pytest.mark.parametrize("op,size", [("spmm_gemm", "small"), ("spmm_gemm", "large"),
                                      ("sddmm_spmm_gemm", "small"), ("sddmm_spmm_gemm", "large")])
 def test_fused_call_routing(slnr, orc, op, size):
-    # the fused call takes the tensor-core kernel from 2^14 nonzeros on (TF32
-    # allowed, supported widths) and the CUDA-core kernels below; both agree
-    # with the oracle
+    # the fused call takes the tensor cores from 2^14 nonzeros on (TF32
+    # allowed, supported widths) and the CUDA cores below, in either order of
+    # the dense product; all agree with the oracle
     n, deg = (1024, 10) if size == "small" else (4000, 12)
     w = wl.spmm_gemm_rmat(0x51A4 + 97, n, deg, 64, 64) if op == "spmm_gemm" else \
         wl.sddmm_spmm_gemm_rmat(0x51A4 + 98, n, deg, 64, 64, 64)
     nnz = len(w.B.crd)
     assert (nnz < (1 << 14)) == (size == "small")
-    slnr.timing_enable(True)
-    try:
-        check(slnr, orc, w, "fused", True)
-        names = [name for name, _ in slnr.timing_read()]
-        launches = slnr.timing_launches()
-    finally:
-        slnr.timing_enable(False)
-    on_tc = any(name.startswith("tc_") for name in names)
-    assert on_tc == (size == "large"), names
+    ref, ref_abs = orc.run(w)
+    sums = "flat_sum" if op == "spmm_gemm" else "flat_sddmm_spmm"
+    got, names = P.phases(w, allow_tf32=True)
+    launches = slnr.timing_launches()
+    assert names == ["tc_premul" if size == "large" else "premul", "flat_rows", sums]
+    assert P.rel_err(got.cpu().numpy(), ref, ref_abs) <= P.TOL_TF32
     # every phase launches at least one kernel; none launches more than two
+    assert len(names) <= launches <= 2 * len(names), (names, launches)
+    names = P.check_row_first(w, True, ref, ref_abs, P.TOL_TF32)
+    launches = slnr.timing_launches()
+    chunks = "spmm" if op == "spmm_gemm" else "sddmm_spmm"
+    assert names == (["seg_count", "seg_write", f"tc_{op}", "combine"] if size == "large" else
+                     ["classify", f"{chunks}_chunks", f"{op}_tiles", "combine"])
     assert len(names) <= launches <= 2 * len(names), (names, launches)
 
 

@@ -42,6 +42,8 @@ def check(slnr, orc, w, variant="fused", allow_tf32=False):
     err = P.rel_err(out.cpu().numpy(), ref, ref_abs)
     tol = P.tolerance(w.op, allow_tf32, variant)
     assert err <= tol, f"{w.name} {variant} tf32={allow_tf32}: err {err:.3e} > {tol:.1e}"
+    if variant == "fused" and w.op in P.GATHERED:
+        P.check_row_first(w, allow_tf32, ref, ref_abs, tol)
     return out
 
 
@@ -72,8 +74,9 @@ def test_mttkrp_gemm_widths(slnr, orc, L, M, variant):
 @pytest.mark.parametrize("L,M", [(4, 8), (32, 64), (256, 16)])
 @pytest.mark.parametrize("variant", ["fused", "unfused"])
 def test_mttkrp_gemm_hub_slice(slnr, orc, L, M, variant):
-    # 3 slices of more than 16 units (two-level sums, the largest in 3 runs of
-    # at most 64 units), 37 small ones (a warp each)
+    # unfused: 3 slices of more than 16 units (two-level sums, the largest in 3
+    # runs of at most 64 units), 37 small ones (a warp each); fused: slices of
+    # hundreds of windows, of a few and of one
     w = wl.mttkrp_gemm_zipf(0x51A5, (40, 400, 500), 150000, 1.8, L, M)
     check(slnr, orc, w, variant, False)
     check(slnr, orc, w, variant, True)
@@ -113,7 +116,7 @@ def test_no_nonzeros(slnr, orc, op, variant):
 @pytest.mark.parametrize("op", ["sddmm_spmm_gemm", "spmmh_gemm"])
 @pytest.mark.parametrize("variant", ["fused", "unfused"])
 def test_rows_at_the_split_thresholds(slnr, orc, op, variant):
-    # 127/128/129 straddle the tensor-core segment length, 255/256/257 the
+    # row first: 127/128/129 straddle the segment length, 255/256/257 the
     # light/heavy boundary of the row kernels, 5000 is a long heavy row; a
     # ragged number of rows (not a multiple of any tile)
     lens = [127, 128, 129, 255, 256, 257, 5000, 1, 0, 3] + [0] * 35

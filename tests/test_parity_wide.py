@@ -5,8 +5,8 @@ Powers of two in [4, 256] run on the specialised kernels (K = 256 with
 L <= 64 on the tensor cores); other widths run on the run-time-width kernels
 with the same schedules.  Each expression is checked element by element at
 widths past 256, at widths that are not powers of two, and at mixed pairs,
-in both variants and both contraction precisions, on inputs with heavy rows
-(split into chunks) and ragged row tiles.  Widths outside the contract (not
+in both variants, both contraction precisions and both orders of the dense
+product, on inputs with heavy rows (split into chunks) and ragged row tiles.  Widths outside the contract (not
 a multiple of 4, or above 1024) are rejected before any launch.
 """
 import ctypes
@@ -45,6 +45,8 @@ def check(slnr, orc, w, variant, allow_tf32):
     err = P.rel_err(P.values_of(w.op, out).cpu().numpy(), ref, ref_abs)
     tol = P.tolerance(w.op, allow_tf32, variant)
     assert err <= tol, f"{w.name} {w.dims} {variant} tf32={allow_tf32}: err {err:.3e} > {tol:.1e}"
+    if variant == "fused" and w.op in P.GATHERED:
+        P.check_row_first(w, allow_tf32, ref, ref_abs, tol)
 
 
 VARIANTS = [("fused", False), ("fused", True), ("unfused", False), ("unfused", True)]

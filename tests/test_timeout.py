@@ -1,11 +1,12 @@
 """Failure detection: a bounded device-side wait that gives up is reported.
 
-The tensor-core kernel's waits (on its mbarriers, its shared counters and its
-tile-index ring) give up after slnr_set_wait_limit cycles.  With a limit far
-below the time a tile takes to build, the MMA warp's first wait for a full
-tile runs out: the kernel sets the timeout bit of the workspace flag word,
-drains the MMAs it issued (with the default limit) and frees its tensor
-memory, and a call in validate mode returns SLNR_ERR_TIMEOUT.  Nothing here
+The waits of the two tensor-core kernels (the row kernel's on its mbarriers,
+its shared counters and its tile-index ring, the product's on its mbarriers)
+give up after slnr_set_wait_limit cycles.  With a limit far below the time a
+tile or a chunk takes to build, the MMA warp's first wait for one runs out: the
+kernel sets the timeout bit of the workspace flag word, drains the MMAs it
+issued (with the default limit) and frees its tensor memory, and a call in
+validate mode returns SLNR_ERR_TIMEOUT.  Nothing here
 faults or hangs the GPU: every wait ends, and the context stays usable, which
 the correct call after the timeout checks against the oracle.
 """
@@ -41,10 +42,14 @@ def test_wait_limit_rejects_negative():
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("kernel", ["tc_premul", "tc_spmm_gemm"])
 @pytest.mark.parametrize("op", ["spmm_gemm", "spttm_ttm"])
-def test_short_wait_limit_reports_timeout(slnr, op):
+def test_short_wait_limit_reports_timeout(slnr, op, kernel):
     w = wl.spmm_gemm_rmat(0x51A4 + 77, 6000, 16, 64, 64) if op == "spmm_gemm" else \
         wl.spttm_ttm_powerlaw(0x51A4 + 78, (200, 200, 900), 60000, 8.0, 900, 64, 64)
+    if kernel == "tc_spmm_gemm":
+        w = P.row_first(w)
+    assert kernel in P.phases(w, allow_tf32=True)[1]
     B, dense = P.to_device(w)
     lib = slnr.lib()
     assert lib.slnr_set_wait_limit(ctypes.c_int64(1000)) == 0
