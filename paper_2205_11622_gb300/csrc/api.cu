@@ -667,7 +667,7 @@ slnr_status sddmm_spmm(const slnr_csr* B, const float* C, const float* D, int32_
   SLNR_LAUNCH("classify", launch_classify(v, sp, s));
   if (!all_pow2(L, K)) {
     float* Y = reinterpret_cast<float*>(ws + l.o_inter);
-    SLNR_LAUNCH("w_sddmm", launch_w_sddmm_spmm(v, C, D, L, nullptr, K, nullptr, Y, sp, s));
+    SLNR_LAUNCH("w_sddmm", launch_w_sddmm_spmm(v, C, D, L, nullptr, K, Y, sp, s));
     CsrView vy = v;
     vy.vals = Y;
     SLNR_LAUNCH("w_spmm", launch_w_spmm(K, vy, E, nullptr, A, sp, s));
@@ -1061,13 +1061,13 @@ slnr_status slnr_sddmm_spmm_gemm(const slnr_csr* B, const float* C, const float*
   SLNR_LAUNCH("classify", launch_classify(v, sp, s));
   if (!all_pow2(K, L, M)) {
     if (opts->variant == SLNR_FUSED) {
-      SLNR_LAUNCH("w_sddmm_spmm_chunks", launch_w_sddmm_spmm(v, C, D, K, F, L, nullptr, nullptr, sp, s));
+      SLNR_LAUNCH("w_sddmm_spmm_chunks", launch_w_sddmm_spmm(v, C, D, K, F, L, nullptr, sp, s));
       SLNR_LAUNCH("w_sddmm_spmm_gemm_tiles", launch_w_sddmm_spmm_gemm_tiles(v, C, D, K, F, L, W, M, A, s));
       SLNR_LAUNCH("w_combine", launch_w_combine(L, sp, W, M, A, s));
     } else {
       float* Y = reinterpret_cast<float*>(ws + l.o_inter);
       float* T = reinterpret_cast<float*>(ws + l.o_inter2);
-      SLNR_LAUNCH("w_sddmm", launch_w_sddmm_spmm(v, C, D, K, nullptr, L, nullptr, Y, sp, s));
+      SLNR_LAUNCH("w_sddmm", launch_w_sddmm_spmm(v, C, D, K, nullptr, L, Y, sp, s));
       CsrView vy = v;
       vy.vals = Y;
       SLNR_LAUNCH("w_spmm", launch_w_spmm(L, vy, F, nullptr, T, sp, s));

@@ -167,7 +167,7 @@ cudaError_t launch_slices_times(const slnr_csf3& B, int L, int M, const float* U
 
 // sddmm.cu
 // fused <SDDMM,SpMM>: the heavy rows' chunks (partials) and the light rows in
-// one launch (plan.hdr->next_row must be 0: warps take work from it)
+// one launch (plan.hdr->next_row must be 0: warps take work from it); L and K up to 64
 cudaError_t launch_sddmm_spmm_rows(const CsrView& B, const float* C, const float* D, int L,
                                    const float* E, int K, float* A, const SplitPlan& plan, cudaStream_t s);
 cudaError_t launch_sddmm_spmm_chunks(const CsrView& B, const float* C, const float* D, int L,
@@ -214,10 +214,10 @@ cudaError_t launch_w_combine(int W, const SplitPlan& plan, const float* D, int L
 cudaError_t launch_w_spmm_gemm_tiles(int K, int L, const CsrView& B, const float* C, const float* C2,
                                      const float* D, float* A, cudaStream_t s);
 cudaError_t launch_w_dense_gemm(int64_t M, int K, int L, const float* T, const float* D, float* A, cudaStream_t s);
-// fused <SDDMM,SpMM> (C nrows x Kd, D ncols x Kd, E ncols x Ko): light rows to A,
-// heavy rows' chunks to plan.partial; with Y not NULL, only the sampled products Y[p]
+// sampled rows (C nrows x Kd, D ncols x Kd, E ncols x Ko): heavy rows' chunks to
+// plan.partial; with Y not NULL, only the sampled products Y[p] of every nonzero
 cudaError_t launch_w_sddmm_spmm(const CsrView& B, const float* C, const float* D, int Kd, const float* E, int Ko,
-                                float* A, float* Y, const SplitPlan& plan, cudaStream_t s);
+                                float* Y, const SplitPlan& plan, cudaStream_t s);
 cudaError_t launch_w_sddmm_spmm_gemm_tiles(const CsrView& B, const float* C, const float* D, int K, const float* F,
                                            int L, const float* W, int M, float* A, cudaStream_t s);
 // unfused MTTKRP: unit partials from the per-fiber T

@@ -335,8 +335,11 @@ cudaError_t launch_sddmm_spmm_rows(const CsrView& B, const float* C, const float
   const int64_t cap = (int64_t)device_sm_count() * SLNR_SDDMM_MIN_CTAS;
   if (ctas > cap) ctas = cap;
   SLNR_WIDTH_SWITCH(WM, W, {
-    k_sddmm_spmm_rows<W><<<SLNR_COUNTED((unsigned)ctas), 256, 0, s>>>(plan.hdr, B.nrows, B.pos, B.crd, B.vals, C, D, L, E, K, A,
-                                                         plan.chunks, plan.max_chunks, plan.partial);
+    if constexpr (W <= 64)  // wider rows run on the windows (flat.cu)
+      k_sddmm_spmm_rows<W><<<SLNR_COUNTED((unsigned)ctas), 256, 0, s>>>(plan.hdr, B.nrows, B.pos, B.crd, B.vals, C, D, L, E,
+                                                           K, A, plan.chunks, plan.max_chunks, plan.partial);
+    else
+      return cudaErrorInvalidValue;
   });
   return cudaGetLastError();
 }

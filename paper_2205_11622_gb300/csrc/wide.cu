@@ -343,10 +343,9 @@ __device__ __forceinline__ void w_stage_row(float* cs, const float* __restrict__
   __syncwarp();
 }
 
-// Fused <SDDMM,SpMM> (A(i,:) = sum_j B(i,j) <C(i,:), D(j,:)> E(j,:)): a warp
-// per item, heavy-row chunks first (partial rows of width Ko), then light
-// rows (A rows written once; with A NULL, the chunks only).  With Y not NULL:
-// the unfused first step, the sampled products Y[p] for every nonzero.
+// Sampled rows, a warp per item.  With Y NULL: the chunks of heavy rows, each
+// partial row sum_j B(i,j) <C(i,:), D(j,:)> E(j,:) (width Ko).  With Y: the
+// unfused first step, the sampled products Y[p] of every nonzero, chunks first.
 template <int NCH>
 __global__ void __launch_bounds__(kWThreads) k_w_sddmm_spmm(const WsHeader* __restrict__ hdr, int nrows,
                                                             const int32_t* __restrict__ pos,
@@ -354,14 +353,14 @@ __global__ void __launch_bounds__(kWThreads) k_w_sddmm_spmm(const WsHeader* __re
                                                             const float* __restrict__ vals,
                                                             const float* __restrict__ C, const float* __restrict__ D,
                                                             int Kd, const float* __restrict__ E, int Ko,
-                                                            float* __restrict__ A, const Chunk* __restrict__ chunks,
-                                                            int max_chunks, float* __restrict__ partial,
+                                                            const Chunk* __restrict__ chunks, int max_chunks,
+                                                            float* __restrict__ partial,
                                                             float* __restrict__ Y) {
   extern __shared__ float4 wsm4[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   float* cs = reinterpret_cast<float*>(wsm4) + (size_t)wib * Kd;
   const int nch = min(hdr->n_chunks, max_chunks);
-  const int64_t nitems = (int64_t)nch + (A != nullptr || Y != nullptr ? nrows : 0);  // A, Y NULL: the chunks only
+  const int64_t nitems = (int64_t)nch + (Y != nullptr ? nrows : 0);
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nitems; w += nwarps) {
     float4 acc[NCH];
@@ -377,7 +376,6 @@ __global__ void __launch_bounds__(kWThreads) k_w_sddmm_spmm(const WsHeader* __re
       if (p1 - p0 > kLightMax) continue;  // its chunks above
       w_stage_row(cs, C, r, Kd, lane);
       w_sddmm_row<NCH>(acc, cs, p0, p1, crd, vals, D, Kd, E, Ko, Y, lane);
-      if (Y == nullptr) wstore(A + r * Ko, acc, Ko, lane);
     }
   }
 }
@@ -577,7 +575,7 @@ cudaError_t launch_w_dense_gemm(int64_t M, int K, int L, const float* T, const f
 }
 
 cudaError_t launch_w_sddmm_spmm(const CsrView& B, const float* C, const float* D, int Kd, const float* E, int Ko,
-                                float* A, float* Y, const SplitPlan& plan, cudaStream_t s) {
+                                float* Y, const SplitPlan& plan, cudaStream_t s) {
   if (B.nrows <= 0) return cudaSuccess;
   const size_t smem = sizeof(float) * (kWThreads / 32) * (size_t)Kd;
   const int wmax = Kd > Ko ? Kd : Ko;
@@ -585,7 +583,7 @@ cudaError_t launch_w_sddmm_spmm(const CsrView& B, const float* C, const float* D
     cudaError_t e = w_smem(k_w_sddmm_spmm<NC>, smem);
     if (e != cudaSuccess) return e;
     k_w_sddmm_spmm<NC><<<SLNR_COUNTED(w_grid((int64_t)B.nrows + plan.max_chunks)), kWThreads, smem, s>>>(
-        plan.hdr, B.nrows, B.pos, B.crd, B.vals, C, D, Kd, E, Ko, A, plan.chunks, plan.max_chunks, plan.partial, Y);
+        plan.hdr, B.nrows, B.pos, B.crd, B.vals, C, D, Kd, E, Ko, plan.chunks, plan.max_chunks, plan.partial, Y);
   });
   return cudaGetLastError();
 }
