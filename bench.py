@@ -177,23 +177,34 @@ def consumer_flops(w) -> int:
     return 0
 
 
-def gather_bytes(w, product_first=False) -> int:
-    """Bytes the fused kernels read as whole gathered rows, one (or two)
-    per nonzero and one per fiber where a fiber scales a row: nnz 4K for
-    <SpMM,GEMM>, nnz 4L for <SpTTM,SpTTM>, nnz 8J for <SpMMH,GEMM>, nnz 4(L+K)
-    for <SDDMM,SpMM>, nnz 4(K+L) for <SDDMM,SpMM,GEMM>, (nnz + nfibers) 4L for
-    MTTKRP.  Where the dense product comes first (product_first), a row of that
-    product takes the place of the gathered operands: nnz 4L, or 4M for
-    <SpTTM,SpTTM>.  Almost all of them hit in L2; their rate, not HBM's, is the
-    realistic ceiling of the gathering kernels."""
-    d, B = w.dims, w.B
-    if product_first:
-        return int(4 * d["M" if w.op == "spttm_ttm" else "L"] * B.nnz)
-    per_nnz = {"spmm_gemm": lambda: 4 * d["K"], "spttm_ttm": lambda: 4 * d["L"], "spmmh_gemm": lambda: 8 * d["J"],
-               "sddmm_spmm": lambda: 4 * (d["L"] + d["K"]), "sddmm_spmm_gemm": lambda: 4 * (d["K"] + d["L"]),
-               "mttkrp": lambda: 4 * d["L"], "mttkrp_gemm": lambda: 4 * d["L"]}[w.op]()
-    extra = 4 * d["L"] * B.nfibers if w.op in ("mttkrp", "mttkrp_gemm") else 0
-    return int(per_nnz * B.nnz + extra)
+def product_order(phases) -> str:
+    """How a call with these phases orders its dense matrices: their product first ("product"), the Hadamard product of
+    the gathered matrices first ("hadamard"), or row by row ("rows")."""
+    if "tc_premul" in phases or "premul" in phases:
+        return "product"
+    return "hadamard" if "hadamard" in phases else "rows"
+
+
+def gathered_widths(w, order="rows"):
+    """Widths (fp32 values) of the whole rows that the fused kernels read per nonzero; the last is the one summed."""
+    d = w.dims
+    rows = {"spmm_gemm": ["K"], "spttm_ttm": ["L"], "spmmh_gemm": ["J", "J"], "sddmm_spmm": ["L", "K"],
+            "sddmm_spmm_gemm": ["K", "L"], "mttkrp": ["L"], "mttkrp_gemm": ["L"]}
+    product = {"spmm_gemm": ["L"], "spttm_ttm": ["M"], "spmmh_gemm": ["L"], "sddmm_spmm_gemm": ["K", "M"]}
+    names = ["J"] if order == "hadamard" else product[w.op] if order == "product" else rows[w.op]
+    return [d[n] for n in names]
+
+
+def gather_bytes(w, order="rows") -> int:
+    """Bytes the fused kernels read as whole gathered rows, one or two per
+    nonzero (gathered_widths) and one per fiber where a fiber scales a row:
+    row by row nnz 4K for <SpMM,GEMM>, nnz 4L for <SpTTM,SpTTM>, nnz 8J for
+    <SpMMH,GEMM>, nnz 4(L+K) for <SDDMM,SpMM>, nnz 4(K+L) for
+    <SDDMM,SpMM,GEMM>, (nnz + nfibers) 4L for MTTKRP.  Almost all of them hit
+    in L2; their rate, not HBM's, is the realistic ceiling of the gathering
+    kernels."""
+    extra = 4 * w.dims["L"] * w.B.nfibers if w.op in ("mttkrp", "mttkrp_gemm") else 0
+    return int(4 * sum(gathered_widths(w, order)) * w.B.nnz + extra)
 
 
 def dense_product_shape(w):
@@ -203,14 +214,11 @@ def dense_product_shape(w):
             "spttm_ttm": lambda: (d["L"], d["M"]), "sddmm_spmm_gemm": lambda: (d["L"], d["M"])}[w.op]()
 
 
-def gather_row_width(w) -> int:
-    """Width (fp32 values) of the rows the producers gather, as a power of two
+def gather_row_width(w, order="rows") -> int:
+    """Width (fp32 values) of the rows that the kernels sum, as a power of two
     in [4, 128] for the gather peak kernel."""
-    d = w.dims
-    width = {"spmm_gemm": "K", "spttm_ttm": "L", "spmmh_gemm": "J", "sddmm_spmm": "K", "sddmm_spmm_gemm": "L",
-             "mttkrp": "L", "mttkrp_gemm": "L"}[w.op]
     v = 4
-    while v * 2 <= min(d[width], 128):
+    while v * 2 <= min(gathered_widths(w, order)[-1], 128):
         v *= 2
     return v
 
@@ -568,8 +576,9 @@ def main():
     achieved = mbytes[dom] / (k_ms / 1e3) / 1e9
     all_rows = min_bytes_all_rows(dw)
     traffic = ncu_traffic(dw.name)
-    pk = slnr.peaks(stream, gather_width=gather_row_width(dw)) if rank == 0 else {}
-    gb = gather_bytes(dw, product_first=kname == "flat_sum")
+    order = product_order(kern_ms[dom])
+    pk = slnr.peaks(stream, gather_width=gather_row_width(dw, order)) if rank == 0 else {}
+    gb = gather_bytes(dw, order)
     cflops, c_ms = consumer_flops(dw), k_ms
     for name in ("tc_premul", "premul"):  # the dense product first: once per column, in a launch of its own
         if name in kern_ms[dom]:
@@ -597,7 +606,7 @@ def main():
                            "hbm_gather_peak_measured": round(pk.get("hbm_gather_gbs", 0.0), 1),
                            "frac_l2": round(gb / (k_ms / 1e3) / 1e9 / pk["l2_gather_gbs"], 4)
                            if pk.get("l2_gather_gbs") else None,
-                           "row_width": gather_row_width(dw),
+                           "row_width": gather_row_width(dw, order),
                            "note": "whole rows the dominant kernel gathers (one or two per nonzero), against "
                                    "this library's own row-gather kernel on an L2-resident table (a quarter "
                                    "of L2) and on a 2 GB table"}}

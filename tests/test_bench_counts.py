@@ -145,3 +145,21 @@ def test_gather_row_width_is_a_power_of_two_up_to_128(width, want):
     B = wl.CSR(2, 2, np.asarray([0, 1, 1], np.int32), np.asarray([1], np.int32), np.ones(1, np.float32))
     w = wl.Workload("w", "spmm_gemm", B, {}, {"K": width, "L": 8})
     assert bench.gather_row_width(w) == want
+
+
+@pytest.mark.parametrize("op,dims,phases,widths,row", [
+    ("spmm_gemm", {"K": 64, "L": 16}, ["seg_count", "tc_spmm_gemm"], [64], 64),
+    ("spmm_gemm", {"K": 64, "L": 16}, ["tc_premul", "flat_rows", "flat_sum"], [16], 16),
+    ("spttm_ttm", {"L": 128, "M": 32}, ["copy_levels", "premul", "flat_sum"], [32], 32),
+    ("spmmh_gemm", {"J": 64, "L": 16}, ["seg_count", "tc_spmmh_gemm"], [64, 64], 64),
+    ("spmmh_gemm", {"J": 64, "L": 16}, ["seg_count", "hadamard", "tc_spmm_gemm"], [64], 64),
+    ("spmmh_gemm", {"J": 64, "L": 16}, ["tc_premul", "flat_sum"], [16], 16),
+    ("sddmm_spmm_gemm", {"K": 64, "L": 64, "M": 16}, ["tc_sddmm_spmm_gemm"], [64, 64], 64),
+    ("sddmm_spmm_gemm", {"K": 32, "L": 64, "M": 16}, ["premul", "flat_sddmm_spmm"], [32, 16], 16)])
+def test_gathered_rows_follow_the_order_taken(op, dims, phases, widths, row):
+    B = wl.CSR(2, 2, np.asarray([0, 1, 3], np.int32), np.asarray([1, 0, 1], np.int32), np.ones(3, np.float32))
+    w = wl.Workload("w", op, B, {}, dims)
+    order = bench.product_order(phases)
+    assert bench.gathered_widths(w, order) == widths
+    assert bench.gather_bytes(w, order) == 4 * 3 * sum(widths)
+    assert bench.gather_row_width(w, order) == row
