@@ -51,6 +51,15 @@ constexpr int flat_ctas() {
   return NCH == 1 ? (MODE == kSum ? kFlatCtas : kFlatCtas2) : NCH == 2 ? 4 : 2;
 }
 
+// Rows of pos that a lane holds: a group looks at 8 rows a step (4 where it is
+// one lane), or windows of short rows wait for pos again and again
+// (<SDDMM,SpMM> 16/16 on R-MAT graphs of 30k rows, degrees 8 and 32: one row a
+// lane 43 and 50 us, four 37 and 44; row kernel 31 and 41).
+template <int GS>
+constexpr int flat_look() {
+  return GS >= 8 ? 1 : GS == 4 ? 2 : 4;
+}
+
 // Largest r in [lo, n) with pos[r] <= p, given lo < n and pos[lo] <= p; one
 // thread.  The row is near lo as a rule: kProbe loads in flight first double
 // the distance until a row lies past p, then cut the rows that are left by
@@ -264,6 +273,7 @@ __global__ void __launch_bounds__(kFlatThreads, flat_ctas<NCH, MODE>()) k_flat(c
   constexpr int NS = kStage / GPW;  // nonzeros of a window per stage
   constexpr int U0 = flat_u<NCH, MODE>();
   constexpr int U = NS < U0 ? NS : U0;
+  constexpr int NB = flat_look<GS>();
   constexpr unsigned FULL = 0xffffffffu;
   static_assert(NS % U == 0 && NS == 2 * GS, "batches tile a stage");
   __shared__ __align__(16) FlatStage stage[kFlatThreads / 32];
@@ -295,11 +305,14 @@ __global__ void __launch_bounds__(kFlatThreads, flat_ctas<NCH, MODE>()) k_flat(c
   int p = (int)(w * a.win < a.nnz ? w * a.win : a.nnz);  // first nonzero of the window's stage
   const int p1 = (int)((int64_t)p + a.win < a.nnz ? p + a.win : a.nnz);
   int rnext = p < p1 ? a.first[w] : a.nrows;  // rows before it start before nonzero p
-  int b, b1;             // pos[rnext + gl], pos[rnext + gl + 1], loaded ahead
+  // pos of rows rnext + NB gl, ..., loaded ahead: NB rows a lane and the one after
+  int b[NB + 1];
   auto peek = [&]() {
-    const unsigned r = item(rnext, gl);
-    b = r < (unsigned)a.nrows ? __ldg(a.pos + r) : INT_MAX;
-    b1 = r < (unsigned)a.nrows ? __ldg(a.pos + r + 1) : INT_MAX;
+#pragma unroll
+    for (int j = 0; j <= NB; ++j) {
+      const unsigned r = item(rnext, NB * gl + j);
+      b[j] = r < (unsigned)a.nrows ? __ldg(a.pos + r) : INT_MAX;
+    }
   };
   peek();
   int cur = -1;               // the row being summed
@@ -307,7 +320,7 @@ __global__ void __launch_bounds__(kFlatThreads, flat_ctas<NCH, MODE>()) k_flat(c
   R acc, c;                   // c: C's row of `cur` (kSampled)
   acc.zero();
   if constexpr (MODE == kSampled) c.load(m.c, (uint32_t)(rnext < a.nrows ? rnext : 0));
-  if (__shfl_sync(FULL, b, g * GS) < p) {  // the window starts inside row rnext
+  if (__shfl_sync(FULL, b[0], g * GS) < p) {  // the window starts inside row rnext
     cur = rnext;
     dst = typename R::Ptr(a.head, a.W, gl).row((uint32_t)w);
   }
@@ -322,19 +335,32 @@ __global__ void __launch_bounds__(kFlatThreads, flat_ctas<NCH, MODE>()) k_flat(c
     }
     __syncwarp();
     fetch(s + NS);
-    // mark the rows that start in [p, pe): GS rows of pos per group and step
+    // mark the rows that start in [p, pe): NB GS rows of pos per group and step
     const int pe = step_end(p, NS, p1);
     bool more = p < pe;
     do {
-      const bool in = more && b < pe, full = in && b1 > b && b >= p;
-      if (full) st.row[g * NS + b - p] = rnext + gl;
-      const unsigned mi = __ballot_sync(FULL, in) & gmask, mf = __ballot_sync(FULL, full) & gmask;
-      rnext += __popc(mi);
-      more = more && mi == gmask;
-      if (more && mf == 0 && rnext < a.nrows) {  // empty rows: on to the row with the next nonzero
+      int rows = 0;  // of this lane that start before pe
+      bool mark = false;
+#pragma unroll
+      for (int j = 0; j < NB; ++j) {
+        const bool in = more && b[j] < pe, full = in && b[j + 1] > b[j] && b[j] >= p;
+        if (full) st.row[g * NS + b[j] - p] = rnext + NB * gl + j;
+        rows += in;
+        mark |= full;
+      }
+      const unsigned marked = __ballot_sync(FULL, mark) & gmask;
+      if constexpr (NB == 1) {
+        rows = __popc(__ballot_sync(FULL, rows != 0) & gmask);
+      } else {
+#pragma unroll
+        for (int o = GS / 2; o > 0; o >>= 1) rows += __shfl_xor_sync(FULL, rows, o);
+      }
+      rnext += rows;
+      more = more && rows == NB * GS;
+      if (more && marked == 0 && rnext < a.nrows) {  // empty rows: on to the row with the next nonzero
         rnext = row_of(a.pos, rnext, a.nrows, __ldg(a.pos + rnext));  // never back: every step passes a row
       }
-      if (mi != 0) peek();
+      if (rows != 0) peek();
     } while (__any_sync(FULL, more));
     __syncwarp();
     const unsigned long long marks = (unsigned long long)__ballot_sync(FULL, st.row[lane] >= 0) |
