@@ -342,15 +342,15 @@ enum PremulKind { kOne, kTwo, kSampledRows, kFibers };
 // the whole result that grows with the longest row's share: up to 5 such
 // deviations times the root of (longest row / mean row).  D first is left to
 // calls where that stays below 2e-2: fibers that cannot be 350 (175) times as
-// long as the mean one, and graphs of fewer than 128k (64k) rows.  Largest
+// long as the mean one, and graphs of fewer than 128k (16k) rows.  Largest
 // difference of any value over the result's rms (or over itself where that is
-// larger), R-MAT graphs, 24 to 300 inputs each: under 128k rows 0.0137 (fp32,
-// under 64k rows, 0.0124); 250k 0.0207, 520k 0.0215, 1M 0.028; 5000-long modes
-// of fibers of mean 8 0.0246, modes of up to 2800 0.0110.
+// larger), R-MAT graphs, 24 to 700 inputs each: under 128k rows 0.0137, 250k
+// 0.0207, 520k 0.0215, 1M 0.028 (product in fp32: 34k 0.0188, under 16k
+// 0.0066); fibers of mean 8 in modes of 5000 0.0246, of up to 2800 0.0115.
 bool premul_near(PremulKind kind, int64_t nrows, int64_t ncols, int64_t nnz, int32_t K, int32_t L) {
   const bool rounded = tc_split_supported(K, L);
   if (kind == kFibers) return ncols * nrows <= (rounded ? 350 : 175) * nnz;
-  return nrows < (rounded ? 128 : 64) * 1024;
+  return nrows < (rounded ? 128 : 16) * 1024;
 }
 
 // Whether the columns that X has more than B has rows are worth their share of
