@@ -317,12 +317,15 @@ bool use_tc_fused(const slnr_opts* o, int32_t K, int32_t L, int64_t nnz) {
 //  - fp32, or widths without a tensor-core row kernel: D first throughout
 //    (150k rows 64/32 295 | 110, 50k rows 100/48 148 | 71, 500k 64/64 588 |
 //    246), unless D widens the rows more than four times on a call of some
-//    size (uniform 220k rows 12/256 158 | 307);
+//    size (uniform 220k rows 12/256 158 | 307), or at all where the wider rows
+//    are a large part of L2 and gathered many times: R-MAT graphs still gain
+//    there (2.1M nonzeros 32/100 1.5 times), uniform ones lose more (264k rows
+//    64/200 436 | 698, 397k 32/128 287 | 433, 726k 64/128 882 | 1060);
 //  - fibers (<SpTTM,SpTTM>): D first (20M nonzeros 64/64 712 | 430, 1M 156 |
 //    82), unless D widens the rows more than twice and the tensor cores take a
 //    large call (2.5M 32/128 119 | 134);
 //  - sampled rows: row first where D widens them (R-MAT 718k rows 16/16/64
-//    825 | 1142, uniform 39k 16/16/128 40 | 48);
+//    825 | 1142, uniform 39k 16/16/128 40 | 48, 72k 32/32/64 75 | 89);
 //  - tensor cores: uniform graphs gain from D first nearly throughout, R-MAT
 //    graphs lose where the rows are narrow or many (heavy rows and long runs of
 //    empty ones), and the sizes do not tell them apart: D first where neither
@@ -380,7 +383,12 @@ bool premul_first(const slnr_opts* o, PremulKind kind, int64_t nrows, int64_t nc
   const int64_t k = 1024;
   if (kind == kFibers) return !row_tc || L <= 2 * K || nnz < 2048 * k;
   if (kind == kSampledRows && L > 2 * K && nrows >= (L > 4 * K ? 0 : 64 * k)) return false;
-  if (!row_tc) return L <= 4 * K || nnz < 256 * k;
+  if (!row_tc) {
+    const int64_t wider = L - (kind == kTwo ? 2 * K : K);
+    if (nnz * wider >= int64_t(1) << 27 && ncols * L >= int64_t(1) << 24) return false;
+    return L <= 4 * K || nnz < 256 * k;
+  }
+  if (kind == kSampledRows && K <= 32 && L > K && nrows >= 40 * k) return false;
   if (L > 2 * K) return nrows < (K <= 16 && kind == kOne ? 40 * k : 64 * k);
   if (kind == kTwo) return true;
   if (kind == kOne && K <= 32 && nrows >= (K <= 16 ? 40 : 64) * k) return false;

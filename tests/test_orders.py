@@ -176,9 +176,13 @@ def test_sampled_gemm_stays_fp32_at_widths_without_a_tensor_core_kernel(gpu, K, 
     ("spttm_ttm", 4096, 1 << 20, 1 << 20, (128, 128), 0, False),      # a long third mode
     ("spmm_gemm", 4096, 16384, 16384 * 8, (64, 64), 0, True),         # few columns more: the sums pay for them
     ("spmm_gemm", 150001, 150001, 2400016, (64, 32), 0, True),
+    ("spmm_gemm", 264179, 264179, 4830566, (64, 200), 0, False),      # wider rows, beyond what L2 holds of them
+    ("spmm_gemm", 726054, 726054, 11070539, (64, 128), 0, False),
+    ("spmmh_gemm", 257990, 257990, 5857089, (128, 200), 0, True),     # one row of 200 for two of 128
+    ("sddmm_spmm_gemm", 71509, 71509, 1451041, (32, 32, 64), 1, False),
     ("spttm_ttm", 2500000, 5000, 20000000, (64, 64), 0, True),
 ])
-def test_many_columns_go_row_first(op, nrows, ncols, nnz, sizes, tf32, first):
+def test_many_columns_and_wider_rows_go_row_first(op, nrows, ncols, nnz, sizes, tf32, first):
     slnr.build()
     assert (csr_bytes(op, nrows, ncols, nnz, sizes, tf32) >= 4 * ncols * sizes[-1]) == first
 
