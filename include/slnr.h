@@ -9,13 +9,13 @@
  * (Sec. 4.2, Algorithm 1) derives: the outer sparse loop (CSR row, or CSF
  * slice / fiber) is shared by the producer and the consumer, the producer
  * fills a small temporary (a scalar or a vector) and the consumer uses it at
- * once, so the intermediate tensor is never written to memory.  Where a vector
+ * once, so the producer's result is not written to memory (but for
+ * <MTTKRP,GEMM>, whose MTTKRP rows go through the workspace).  Where a vector
  * temporary is multiplied by a dense matrix, the library may take the product
- * in the other order, by sizes and widths alone: the dense matrices first, once
- * per gathered row into the workspace, then the sparse sum (the same sums in
- * another order; with infinite or overflowing values the two orders can differ
- * in what is infinite and what is NaN).  Each entry
- * point also has an UNFUSED variant that materialises the intermediate in the
+ * in the other order, by sizes, widths and the workspace's size alone: the dense
+ * matrices first, once per gathered row into the workspace, then the sparse sum
+ * (the same sums in another order; with overflowing values the two orders can
+ * differ in what is infinite and what is NaN).  Each entry point also has an UNFUSED variant that materialises the intermediate in the
  * caller's workspace and runs producer and consumer as separate kernels (the
  * paper's "TACO Separate" baseline, Sec. 6); slnr_spmm_gemm_original runs
  * <SpMM,GEMM> as the perfect loop nest (its "TACO Original").
@@ -76,7 +76,7 @@ typedef enum slnr_status {
 } slnr_status;
 
 typedef enum slnr_variant {
-  SLNR_FUSED = 0,  /* shared outer sparse loop, temporary kept on chip */
+  SLNR_FUSED = 0,  /* shared outer sparse loop, the producer's temporary used at once (see each entry point) */
   SLNR_UNFUSED = 1 /* producer and consumer as separate kernels, intermediate in workspace */
 } slnr_variant;
 

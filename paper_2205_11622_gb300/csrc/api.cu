@@ -455,12 +455,15 @@ Layout layout_spmm_gemm(const slnr_csr* B, int32_t K, int32_t L, const slnr_opts
 }
 
 // Fused <SDDMM,SpMM> runs on the nonzero-window kernels, whatever the widths,
-// but for large calls and short rows at widths of powers of two up to 64:
-// there four or more windows share a warp, short rows start in one or another
-// of them at almost every step, and the row kernel (a lane group per short
-// row) is ahead (us, windows | rows: R-MAT 5.1M nonzeros 64/64 367 | 342,
-// 14.5M 64/32 720 | 652, 117k rows of 3.1 64/64 72 | 66; otherwise 3.7M 64/32
-// 160 | 160, 2.0M 64/64 120 | 133; wider, 4.8M 128/128 327 | 391).
+// but for large calls and short rows at widths of powers of two up to 64, which
+// run on the row kernel (a lane group per short row): there four or more windows
+// share a warp, and short rows start in one or another of them at almost every
+// step.  us, windows | rows, R-MAT: 14.5M nonzeros 64/32 600 | 576, 5.1M 32/32
+// 159 | 147, but 5.1M 64/64 215 | 237, 117k rows of 3.1 64/64 52 | 62 (the line
+// was drawn when the windows' combine took longer: 367 | 342, 72 | 66);
+// otherwise 2.0M 64/64 117 | 129, 3.7M 64/32 190 | 199, 4.8M 128/128 373 | 403;
+// 16/16 of 0.3 to 1.2M nonzeros 37-60 | 31-58 on R-MAT graphs, half the time on
+// uniform ones.
 constexpr int64_t kRowsMinNnz = int64_t(1) << 22;
 bool use_flat_sddmm(int64_t nrows, int64_t nnz, int32_t L, int32_t K) {
   return (nnz < kRowsMinNnz && nnz >= 4 * nrows) || L > 64 || K > 64 || !all_pow2(L, K);

@@ -23,10 +23,11 @@
 // inside the window's warp, tensors of many small slices took up to 1.5 times
 // as long as with the separate launch (37k nonzeros in 6800 slices 89 us).
 //
-// What bounds it: the L1 data pipe (72 % busy in an ncu capture of 10M
-// nonzeros at L = 32; a C-row load of the few groups whose fiber ends costs as
-// much as one of all eight) and the gathers' latency; 8.8 warp instructions per
-// nonzero (19 with 4 columns a lane and a shuffle per value).
+// What bounds it: L1 (72 % busy in an ncu capture of 10M nonzeros at L = 32, its
+// data pipe 67 %; a C-row load of the few groups whose fiber ends costs as much
+// as one of all eight) and the gathers' latency (7.7 warps waiting for loads for
+// each that issues); 8.6 warp instructions per nonzero (19 with 4 columns a lane
+// and a shuffle per value).
 #include "flat.cuh"
 #include "launch.h"
 

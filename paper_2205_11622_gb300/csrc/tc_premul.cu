@@ -19,9 +19,10 @@
 //   4 epilogue warps: tensor memory -> shared memory -> whole row pieces of G.
 // A tile held whole (128 x 128 hi and lo is 128 KB beside D^T's 64 KB) had a
 // single buffer, so loads, MMAs and stores of one tile followed one another.
-// Whole calls, whole tiles | chunks: 1M rows 128/128 with the Hadamard product
-// and 16M nonzeros 1068 | 980 us, without it 957 | 856; 128/32 664 | 549; 100k
-// rows 64/64 99 | 91; 4k rows 16/16 36 | 31.  A step of the ring holds 32
+// Whole calls with the product first, whole tiles | chunks: 1M rows 128/128 with
+// the Hadamard product and 16M nonzeros 1068 | 980 us, without it 957 | 856;
+// 128/32 664 | 549 (calls of that size now go row first); 100k rows 64/64 99 |
+// 91; 4k rows 16/16 36 | 31.  A step of the ring holds 32
 // columns because D^T (64 KB) and the epilogue's pieces (18 KB) leave 128 KB.
 // Every wait is bounded; a wait that gives up sets kErrTimeout, and MMAs in
 // flight are drained before the tensor memory is freed.
