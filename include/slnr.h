@@ -14,11 +14,12 @@
  * temporary is multiplied by a dense matrix, the library may take the product
  * in the other order, by sizes, widths and the workspace's size alone: the dense
  * matrices first, once per gathered row into the workspace, then the sparse sum
- * (the same sums in another order; with overflowing values the two orders can
- * differ in what is infinite and what is NaN).  Each entry point also has an UNFUSED variant that materialises the intermediate in the
- * caller's workspace and runs producer and consumer as separate kernels (the
- * paper's "TACO Separate" baseline, Sec. 6); slnr_spmm_gemm_original runs
- * <SpMM,GEMM> as the perfect loop nest (its "TACO Original").
+ * (the same sums in another order; with infinite or overflowing values the two
+ * orders can differ in what is infinite and what is NaN).  Each entry point also
+ * has an UNFUSED variant that materialises the intermediate in the caller's
+ * workspace and runs producer and consumer as separate kernels (the paper's
+ * "TACO Separate" baseline, Sec. 6); slnr_spmm_gemm_original runs <SpMM,GEMM> as
+ * the perfect loop nest (its "TACO Original").
  *
  * Conventions shared by every entry point
  *  - Every array argument (sparse structure, dense operands, outputs,
