@@ -148,7 +148,7 @@ __device__ __forceinline__ void gather_acc(float (&acc)[VPL], const int32_t* __r
                                            const float* __restrict__ X, int ldx, int col,
                                            const float* __restrict__ X2 = nullptr) {
   int p = p0;
-  for (; p1 - p >= U; p += U) {
+  for (; item(p, U) <= (unsigned)p1; p += U) {
     int c[U];
     float v[U];
 #pragma unroll

@@ -24,7 +24,7 @@
 // and <SDDMM,SpMM> of 0.6M at 100/48 4 to 6 (windows of few nonzeros, whose
 // starts and ends are a larger part).  An ncu capture of the 64/64 call: 13
 // warps on an SM, 6 of them waiting for loads for each that issues, issue slots
-// 32 % used, L1 57 %, L2 40 %; of the sums of rows of 32: 26 warps, 50 %, 59 %, 20 %.
+// 32 % used, L1 57 %, L2 40 %; of the sums of rows of 32: 28 warps, 53 %, 62 %, 21 %.
 #include "flat.cuh"
 #include "launch.h"
 

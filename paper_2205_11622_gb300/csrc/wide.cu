@@ -63,7 +63,7 @@ __device__ __forceinline__ void wgather(float4 (&acc)[NCH], const int32_t* __res
                                         const float* __restrict__ X2, int W, int lane) {
   wzero(acc);
   int p = p0;
-  for (; p1 - p >= 2; p += 2) {
+  for (; item(p, 2) <= (unsigned)p1; p += 2) {
     const int c0 = __ldg(crd + p), c1 = __ldg(crd + p + 1);
     const float v0 = __ldg(vals + p), v1 = __ldg(vals + p + 1);
     float4 x0[NCH], x1[NCH];
