@@ -321,9 +321,9 @@ bool use_tc_fused(const slnr_opts* o, int32_t K, int32_t L, int64_t nnz) {
 //    are a large part of L2 and gathered many times: R-MAT graphs still gain
 //    there (2.1M nonzeros 32/100 1.5 times), uniform ones lose more (264k rows
 //    64/200 436 | 698, 397k 32/128 287 | 433, 726k 64/128 882 | 1060);
-//  - fibers (<SpTTM,SpTTM>): D first (20M nonzeros 64/64 712 | 430, 1M 156 |
-//    82), unless D widens the rows more than twice and the tensor cores take a
-//    large call (2.5M 32/128 119 | 134);
+//  - fibers (<SpTTM,SpTTM>): D first (1M nonzeros 64/64 156 | 82, 20M 712 | 430,
+//    where premul_near allows it), unless D widens the rows more than twice and
+//    the tensor cores take a large call (2.5M 32/128 119 | 134);
 //  - sampled rows: row first where D widens them (R-MAT 718k rows 16/16/64
 //    825 | 1142, uniform 39k 16/16/128 40 | 48, 72k 32/32/64 75 | 89);
 //  - tensor cores: uniform graphs gain from D first nearly throughout, R-MAT
