@@ -363,8 +363,8 @@ def _run(name, B, args, sizes, variant, allow_tf32, validate, workspace, stream)
     v = _VARIANTS.get(variant)
     v = int(variant) if v is None else v
     tf32 = 1 if allow_tf32 else 0
-    shape = (B.nrows, B.ncols, B.nnz) if type(B) is slnr_csr else (*B.dim, B.nnz, B.nslices, B.nfibers)
-    need, buf, short = _ws_bytes(name, shape, sizes, v, tf32), workspace.buf, None
+    shape = (B.nrows, B.ncols, B.nnz) if isinstance(B, slnr_csr) else (*B.dim, B.nnz, B.nslices, B.nfibers)
+    need, buf, short = _ws_bytes(name, shape, sizes, v, tf32), getattr(workspace, "buf", None), None
     if buf is None or buf.numel() < need:
         buf, short = _room(workspace, need)
     o = slnr_opts(v, tf32, 1 if validate else 0, 0, s, buf.data_ptr(), buf.numel())
